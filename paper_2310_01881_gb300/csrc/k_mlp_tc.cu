@@ -21,10 +21,10 @@
 // latency of each tile's per-layer chain; keeping A in TMEM removes the
 // shared-memory activation stores and proxy fences from that chain.
 //
-// Thread r of a warpgroup owns sample row r: it rebuilds the sample, encodes
+// Thread r of a compute warpgroup owns sample row r: it rebuilds the sample, encodes
 // gamma(x) ++ gamma(d) and writes it into its TMEM lane (tcgen05.st 32x32b); after
-// each MMA it reads its row of D (tcgen05.ld 32x32b: warp q of the group owns lanes
-// 32q..32q+31) and writes the next layer's A back into TMEM.  BF16 folds layer 0's
+// each layer's MMAs it reads its row of D (tcgen05.ld 32x32b: warp q of the group owns
+// lanes 32q..32q+31) and writes the next layer's A back into TMEM.  BF16 folds layer 0's
 // bias into its contraction (a weight column against a constant-1 input column) and
 // writes every later layer's FP32 bias into its accumulator with one more K = 16 MMA
 // (three constant-1 input columns of layer 0, still in TMEM, against the bias split
@@ -33,20 +33,27 @@
 // (its scales folded into the weights, its bias through a BF16 MMA); with per-row
 // scales it applies its channel scales and bias with one packed FMA per pair first.
 // The 4-wide head is one more BF16 MMA (16 rows, 4 used) on relu(h) written into the
-// group's D columns; it runs while the group encodes its next tile.  Its accumulator
-// sits in 16 TMEM columns that no layer writes, so its outputs (sigma = softplus,
-// rgb = sigmoid) are read with the next tile's layer-0 accumulator and activated and
-// stored while that tile's last layer's MMAs run.
+// group's D columns.  Its outputs (sigma = softplus, rgb = sigmoid) are read with the
+// next tile's layer-0 accumulator and activated and stored under that tile's layer 2.
 //
-// Several warpgroups per CTA work on different tiles, so one group's epilogue
-// overlaps another's MMA.  Each group's leader warp (warp grp % 4 of the group, so
-// the leader warps run on different SM sub-partitions) issues the group's MMAs
-// converged, one lane elected per instruction, and tracks completion with
-// tcgen05.commit on the group's mbarrier, on which every thread of the group then
-// waits itself.  Every wait is bounded (clock64 deadline); a wait that runs out is
-// ORed over the group at its next barrier, the group records AMNERF_E_TIMEOUT in
-// the status word and leaves its tile loop together, and the CTA still frees its
-// TMEM before returning.
+// A tile's chain is shortened from both ends (4 x 64 BF16 network, 8 views of 800 x 800:
+// network step 12.3 -> 9.5 ms; E4M3 with static scales 12.2 -> 8.6 ms):
+//   - what does not need a row's thread sits in one auxiliary warp per group (the fifth
+//     warpgroup): it stages crossing ids, intervals and rays in shared memory tiles ahead
+//     (cp.async), loads the weights and issues the MMAs.  Staging alone gave 12.3 -> 11.0:
+//     the two dependent loads had cost each tile one to two DRAM latencies, as a load into
+//     registers is waited for before the block that issues it is left.  The issue from
+//     warps of its own, and mbarriers in place of group barriers, gave 11.0 -> 9.5.
+//   - the compute warps encode tile t + 1 while tile t's layers run, and store its input
+//     into TMEM columns that are free by then (see kGroupCols).
+//
+// Several groups per CTA work on different tiles (at most four: TMEM), so one group's
+// epilogue overlaps another's MMAs.  Synchronisation, per group: the compute warps arrive
+// on bar_a when a layer's input is written, and wait on bar_m, which the layer's
+// tcgen05.commit completes; bar_h tracks the head MMAs, bar_w the weights, bar_s the
+// staged crossings.  Every wait is bounded (clock64 deadline): a warp whose wait runs out
+// records AMNERF_E_TIMEOUT in the status word and leaves its loop, the group's other warps
+// run out in turn, and the CTA still frees its TMEM before returning.
 //
 // Encoding: sin/cos(pi 2^k p) at k = 0 and k = 5 come from the SFU after an exact
 // argument reduction; the other octaves follow by the double-angle recurrence
@@ -107,9 +114,9 @@ struct TcLayout {
         w0 = 0;
         wh = w0 + (size_t)w * k0p * es;
         wo = wh + (size_t)(h - 1) * w * kh * es;  // head: 16 x khead BF16 (both precisions)
-        sw = wo + (size_t)16 * khead * 2;
-        bias = sw + (f8 ? (size_t)h * w * 4 : 0);
-        bb = (bias + (size_t)h * w * 4 + 16 + 127) / 128 * 128;  // FP32 biases b_0.. and bo, then bb
+        bias = wo + (size_t)16 * khead * 2;
+        // FP32 biases b_0.. and bo, then bb; E4M3 with per-row scales has sw in its place
+        sw = bb = (bias + (size_t)h * w * 4 + 16 + 127) / 128 * 128;
         const size_t end = bb + (size_t)(f8 ? h : h - 1) * w * kBiasK * 2;
         stride = (end + 127) / 128 * 128;
     }
@@ -142,10 +149,15 @@ uint8_t f2e4m3(float x) {
 }
 
 struct TcShared {
-    uint64_t bar_w[kMaxGroups];
-    uint64_t bar_m[kMaxGroups];
+    uint64_t bar_w[kMaxGroups];      // the leaf's weights
+    uint64_t bar_m[kMaxGroups];      // a layer's MMAs
+    // k_mlp_tc only
+    uint64_t bar_h[kMaxGroups];      // a tile's head MMAs
+    uint64_t bar_a[kMaxGroups];      // a layer's input written by the four compute warps
+    uint64_t bar_s[kMaxGroups];      // the next tiles' crossings staged
     int flag[kMaxGroups];
-    uint32_t next_tile[kMaxGroups];  // dynamic schedule: tile grabbed by the group's thread 0
+    int leaf[kMaxGroups][4];         // leaves of a worker's next tiles (k_mlp_tc)
+    uint32_t next_tile[kMaxGroups];  // dynamic schedule: tile grabbed by the group's leader (k_mlp_tc2)
     uint32_t tmem_base;
 };
 
@@ -177,12 +189,46 @@ __device__ __forceinline__ void crossing_data(const MlpArgs& g, uint32_t id, flo
     }
 }
 
-// TMEM columns per warpgroup: D (accumulator, up to 64 FP32 columns), A (up to 48
-// columns = 96 BF16 features per lane), then the head accumulator (16 columns), which
-// no layer writes: a tile's head result is read during the next tile's layers.
+// TMEM columns per warpgroup (128): D (accumulator, up to 64 FP32 columns), A (48
+// columns), then the head accumulator (16 columns).
+//   BF16: the A columns hold a tile's layer-0 input (96 features, two per column).  A
+//   hidden layer's input takes A columns 0..15 (features 0..31) and the head columns
+//   (features 32..63): the head's result is read with the layer-0 accumulator, before
+//   the first of them is written, and its next accumulation starts after the last of
+//   them has been read.  A columns 16..39 are thus free from the completion of a tile's
+//   layer 0 on and take the next tile's input while this tile's layers run (columns
+//   40..47 hold the constant ones that every layer's bias MMA reads).
+//   E4M3: a hidden layer's input takes A columns 0..15, the layer-0 input (four features
+//   per column) columns 16..39, the constant ones of the static mode 40..47.
 constexpr uint32_t kGroupCols = 128;
 constexpr uint32_t kACol = 64;
 constexpr uint32_t kHeadCol = 112;
+constexpr uint32_t kA0Col8 = 16;  // E4M3: first A column of the layer-0 input
+
+// Keeps the n words of a value computed here from being computed later: pure register
+// arithmetic may otherwise be moved past the volatile waits that follow it.
+template <int N>
+__device__ __forceinline__ void pin(uint32_t (&w)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(w[i]));
+}
+
+// Registers per thread: 128 (groups + 1) threads are launched with 96 each; the compute
+// warpgroups take more and leave the last one the rest (at four groups the whole launch:
+// 4 x 112 + 32 = 5 x 96; fewer groups ask for less than they were launched with).
+constexpr int kComputeRegs = 104, kAuxRegs = 64;
+static_assert(kMaxGroups * kComputeRegs + kAuxRegs <= (kMaxGroups + 1) * 96 && kComputeRegs - 96 <= 96 - kAuxRegs,
+              "the split draws on the launch's registers");
+
+// A group's crossings in shared memory, staged ahead by one of its warps (cpt = crossings
+// per tile, 128 / steps): the interval and the ray of every crossing of two tiles (32 B:
+// t_in, t_out, o, d) and the crossing ids of four (0xffffffff past a leaf's end).  The
+// copies are cp.async: a load into registers is waited for before the block that issued it
+// is left, which cost every group one to two DRAM latencies per tile.
+constexpr int kDataSlots = 2, kIdSlots = 4;
+__host__ __device__ constexpr size_t stage_bytes(int cpt) {
+    return (size_t)cpt * (kDataSlots * 32 + kIdSlots * 4);
+}
 
 // F8 = false: BF16 operands (kind::f16, K = 16 per MMA, 2 features per TMEM column).
 // F8 = true:  E4M3 operands (kind::f8f6f4, K = 32 per MMA, 4 features per column).
@@ -199,35 +245,55 @@ constexpr uint32_t kHeadCol = 112;
 template <int W>
 constexpr int kHiddenFor = W == 64 ? 4 : 2;
 
+// relu of this thread's accumulator row (W FP32 columns at d) as BF16, two per column:
+// features 0..31 to the 16 columns at lo, 32..63 to those at hi (which may lie over the
+// columns read before); in two halves, 32 registers instead of 64.
+template <int W>
+__device__ __forceinline__ void relu_row(uint32_t d, uint32_t lo, uint32_t hi) {
+#pragma unroll
+    for (int h = 0; h < W / 32; ++h) {
+        float v[32];
+        uint32_t pk[16];
+        tmem_ld32(d + 32u * h, v);
+#pragma unroll
+        for (int c = 0; c < 16; ++c) pk[c] = pack_relu_bf16(v[2 * c], v[2 * c + 1]);
+        tmem_st16(h == 0 ? lo : hi, pk);
+    }
+}
+
 // JIT: samples at the stratified jitter's fractions of their strata (g.jitter != 0), else
 // at the midpoints.
+//
+// The tiles of a worker are software-pipelined: while the MMAs of tile t's layers run, its
+// group encodes tile t + 1 (the sample position and the direction under layer 0, the
+// position's octaves 5-9 under layer 1, its octaves 0-4 under the last layer) and stores
+// its input into TMEM piece by piece; the arrivals that end tile t publish it too, so its
+// layer 0 starts as soon as tile t's head has completed.
 template <int W, bool F8, bool ST, int HC, bool JIT>
-__global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n_groups, uint32_t tmem_cols) {
+__global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g, int n_groups, uint32_t tmem_cols) {
     const int hidden = HC > 0 ? HC : g.hidden;  // hidden layers (a compile-time constant when HC > 0)
     constexpr int K0 = (3 + 6 * kLX) + (3 + 6 * kLD);
     constexpr int KI = F8 ? 32 : 16;        // K per MMA instruction
-    constexpr int EPW = F8 ? 4 : 2;         // elements per 32-bit TMEM column
     constexpr int K0P = round_up(F8 ? K0 : K0 + 1, KI);  // BF16: + the bias column
-    static_assert(K0P / EPW <= (int)(kHeadCol - kACol), "layer-0 input does not fit the A columns");
+    static_assert(K0P == 96 && kLX == 10 && kLD == 4, "the layer-0 input's layout");
     static_assert(W <= (int)kACol, "accumulator does not fit the D columns");
     extern __shared__ __align__(1024) uint8_t smem[];
     const TcLayout lay(W, hidden, K0, F8);
     TcShared* sh = reinterpret_cast<TcShared*>(smem + lay.stride * n_groups);
 
-    const int grp = threadIdx.x >> 7;
+    // the warp index through a shuffle, so that the compiler knows what derives from it to
+    // be the same for the whole warp (uniform registers: about 15 fewer per thread)
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);
+    const int grp = warp >> 2;
     const int tig = threadIdx.x & 127;  // row within the tile = TMEM lane
-    const int warp = threadIdx.x >> 5;
     const int q = warp & 3;             // TMEM lane quadrant of this warp
-    const int bar_id = 1 + grp;
-    // the group's leader (MMA issue, waits, weight loads) sits in warp grp % 4 of the
-    // group, so the leaders of the 4 groups run on 4 different SM sub-partitions
-    const bool leader = tig == 32 * (grp & 3);
-    const bool leader_warp = warp == 4 * grp + (grp & 3);  // the leader's warp: issues the MMAs, converged
-
     if (threadIdx.x == 0) {
         for (int i = 0; i < n_groups; ++i) {
             mbar_init(smem_u32(&sh->bar_w[i]), 1);
             mbar_init(smem_u32(&sh->bar_m[i]), 1);
+            mbar_init(smem_u32(&sh->bar_h[i]), 1);
+            mbar_init(smem_u32(&sh->bar_a[i]), 4);
+            mbar_init(smem_u32(&sh->bar_s[i]), 33);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -243,207 +309,171 @@ __global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
 
-    if (grp < n_groups) {
-        uint8_t* wbuf = smem + lay.stride * grp;
-        const uint32_t w_addr = smem_u32(wbuf);
-        const uint32_t bar_w = smem_u32(&sh->bar_w[grp]);
-        const uint32_t bar_m = smem_u32(&sh->bar_m[grp]);
-        const uint32_t lane = (uint32_t)(32 * q) << 16;
-        const uint32_t d_col = tmem + kGroupCols * (uint32_t)grp;  // lane 0: MMA operand addresses
-        const uint32_t a_col = d_col + kACol;
-        const uint32_t d_row = d_col + lane;                          // this warp's lanes
-        const uint32_t a_row = a_col + lane;
-        const float* bias = reinterpret_cast<const float*>(wbuf + lay.bias);
-        // shared-memory descriptors of the first core matrix of W0, W1 and the head; the
-        // start-address field holds address / 16 in 14 bits, and every address here is
-        // below 2^18, so later core matrices are these plus (offset / 16)
-        const uint64_t desc_w0 = sdesc(w_addr + (uint32_t)lay.w0, (uint32_t)K0P * (F8 ? 8u : 16u));
-        const uint64_t desc_wh = sdesc(w_addr + (uint32_t)lay.wh, (uint32_t)lay.kh * (F8 ? 8u : 16u));
-        const uint64_t desc_wo = sdesc(w_addr + (uint32_t)lay.wo, (uint32_t)lay.khead * 16u);
-        const uint64_t desc_bb = sdesc(w_addr + (uint32_t)lay.bb, (uint32_t)kBiasK * 16u);
-        const uint8_t* wall = reinterpret_cast<const uint8_t*>(g.weights);
-        if constexpr (F8 && ST) {
-            // the BF16 constant-1 input columns of the bias MMAs (the K = 16 step at
-            // A columns 40..47, ones at its columns 10..12), which no E4M3 operand
-            // reaches (layer 0 fills A columns 0..23, later layers 0..W/4-1): written once
-            const uint32_t c8[8] = {0u, 0u, 0u, 0u, 0u, pack_bf16(1.0f, 1.0f), pack_bf16(1.0f, 0.0f), 0u};
-            static_assert((kOnesCol - kOnesStep) / 2 == 5, "ones at K-step columns 10..12");
-            tmem_st8(a_row + (uint32_t)(kOnesStep / 2), c8);
-            tmem_st_wait();
-        }
+    // Warpgroups 0 .. n_groups - 1 compute; warp i of the last one serves group i: it stages
+    // the crossings, loads the weights and issues the MMAs, so that nothing of that sits in
+    // the compute warps' serial chain.
+    const int srv = warp - 4 * n_groups;                // >= 0: the group this warp serves
+    const int gi = srv >= 0 ? srv : grp;                // this warp's group
+    const bool used = gi < n_groups;
+    uint8_t* wbuf = smem + lay.stride * gi;
+    const uint32_t bar_w = smem_u32(&sh->bar_w[gi]);
+    const uint32_t bar_m = smem_u32(&sh->bar_m[gi]);
+    const uint32_t bar_h = smem_u32(&sh->bar_h[gi]);
+    const uint32_t bar_a = smem_u32(&sh->bar_a[gi]);
+    const uint32_t bar_s = smem_u32(&sh->bar_s[gi]);
+    const uint32_t d_col = tmem + kGroupCols * (uint32_t)gi;  // lane 0: MMA operand addresses
+    const uint32_t a_col = d_col + kACol;
+    // Tile n of the group has its leaf in leaf_s[n % 4] (-1: no such tile), its crossing ids
+    // in id_s[n % 4] and its intervals and rays in data_s[n % 2].
+    const int cpt = kTileRows >> g.lg_steps;
+    uint8_t* stage = reinterpret_cast<uint8_t*>(sh) + ((sizeof(TcShared) + 15) & ~(size_t)15) + gi * stage_bytes(cpt);
+    float* data_s = reinterpret_cast<float*>(stage);
+    uint32_t* id_s = reinterpret_cast<uint32_t*>(stage + (size_t)cpt * kDataSlots * 32);
+    volatile int* leaf_s = sh->leaf[gi];
+    bool ok = true;  // the same in every thread of a warp
+    // A wait that ran out (about 2 s) ends the warp's loop: it arrives at no barrier any
+    // more, so the others of its group run out too and leave.
+    auto wait = [&](uint32_t bar, uint32_t phase) {
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase));
+        return ok;
+    };
 
-        // ---- tile schedule of this worker (one warpgroup)
-        const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
-        const uint32_t workers = gridDim.x * (uint32_t)n_groups;
-        const uint32_t wid = blockIdx.x * (uint32_t)n_groups + (uint32_t)grp;
-        uint32_t t_stop = t_end, t_step = 1, t_first;
-        if (g.schedule == kSchedInterleaved) {
-            t_first = g.t_begin + wid;
-            t_step = workers;
-        } else if (g.schedule == kSchedDynamic) {
-            if (leader) sh->next_tile[grp] = atomicAdd(g.tile_counter, 1u) + g.t_begin;
-            wg_bar(bar_id);
-            t_first = sh->next_tile[grp];
-        } else {  // contiguous (also each launch of the per-leaf loop)
-            const uint32_t span = t_end > g.t_begin ? t_end - g.t_begin : 0u;
-            const uint32_t per = (span + workers - 1) / workers;
-            t_first = min(g.t_begin + wid * per, t_end);
-            t_stop = min(t_first + per, t_end);
-        }
-        volatile int* flag = &sh->flag[grp];
-        const int ci = tig / g.steps;          // crossing of this row within a tile
-        const int j = tig - ci * g.steps;      // sample of this row within its crossing
-        uint32_t ph_w = 0, ph_m = 0;
-        int cur = -1;
-        bool ok = true;
-        // The head MMA of a tile runs while the group encodes its next tile.  Before that
-        // tile's first MMA only the leader warp waits for it (the head reads D, which
-        // layer 0 overwrites; the other warps see it complete through the layer-0
-        // commit); its result, in columns no layer writes, is read with the layer-0
-        // accumulator and activated and stored while a later layer's MMAs run.
-        bool pending = false;   // head MMA issued, its completion not yet consumed
-        bool have_out = false;  // a head result in TMEM waits to be read
-        bool zpend = false;     // a head result in registers waits to be stored
-        bool head_bad = false;  // the leader warp's wait for a head MMA ran out
-        uint64_t slot_prev = ~0ull, slot_z = ~0ull;
-        uint32_t zr[4] = {0u, 0u, 0u, 0u};
-        auto store_head = [&]() {
-            if (slot_z != ~0ull) {  // 4 x FP16; sigma saturates at the FP16 maximum
-                uint2 o;
-                o.x = pack_f16(fminf(softplus_f(__uint_as_float(zr[0])), 65504.0f), sigmoid_f(__uint_as_float(zr[1])));
-                o.y = pack_f16(sigmoid_f(__uint_as_float(zr[2])), sigmoid_f(__uint_as_float(zr[3])));
-                static_cast<uint2*>(g.slot_out)[slot_z] = o;
-            }
-            zpend = false;
-        };
-        // the whole group waits for the head MMA (a leaf change: it reads the weights)
-        auto head_group_wait = [&]() -> bool {
-            const bool okh = group_wait(bar_m, ph_m, bar_id, flag, leader);
-            ph_m ^= 1u;
-            pending = false;
-            return okh;
-        };
-
-        // software pipeline: the crossing id of the next tile is fetched after the first
-        // MMA of the current tile has been waited for, its interval and ray one layer later
-        int leaf = t_first < t_stop ? leaf_of_tile(g.tile_off, g.n_leaves, t_first) : 0;
-        uint32_t id = t_first < t_stop ? row_crossing(g, leaf, t_first, ci) : 0xffffffffu;
-        float2 xi = make_float2(0.f, 0.f);
-        float ro[3] = {0.f, 0.f, 0.f}, rd[3] = {0.f, 0.f, 0.f};
-        crossing_data(g, id, xi, ro, rd);
-        // the looked-up leaf's tile range and crossing range, kept in registers: they
-        // change only at leaf changes, so a tile's lookup is one load (its crossing id)
-        // instead of a chain of three (the small tables leave L1 under the streaming
-        // loads of the intervals and rays)
-        uint32_t lk_t0 = 0u, lk_t1 = 0u, lk_x0 = 0u, lk_x1 = 0u;
-        auto leaf_ranges = [&](int lf) {
-            lk_t0 = __ldg(g.tile_off + lf);
-            lk_t1 = __ldg(g.tile_off + lf + 1);
-            lk_x0 = __ldg(g.offsets + lf);
-            lk_x1 = __ldg(g.offsets + lf + 1);
-        };
-        if (t_first < t_stop) leaf_ranges(leaf);
-
-        for (uint32_t t = t_first; t < t_stop && ok;) {
-            if (leaf != cur) {
-                if (pending && !(ok = head_group_wait())) break;  // the head MMA still reads the weights
-                wg_bar(bar_id);  // every row is done with the previous leaf's weights and biases
-                if (leader) {
-                    fence_proxy_async();
-                    bulk_load(w_addr, wall + (size_t)leaf * lay.stride, (uint32_t)lay.stride, bar_w);
-                }
-                ok = group_wait(bar_w, ph_w, bar_id, flag, leader);
-                ph_w ^= 1u;
-                if (!ok) break;
-                cur = leaf;
-            }
-            // ---- rebuild the sample of this row and encode it into its TMEM lane (layer-0 A)
-            uint64_t slot = ~0ull;  // 64-bit: rays * cap may exceed 2^32
-            float x[3] = {0.f, 0.f, 0.f}, d[3] = {0.f, 0.f, 0.f};
-            if (id != 0xffffffffu) {
-                const uint32_t ray = div_maxc(g, id);
-                const uint32_t k = id - ray * (uint32_t)g.maxc;
-                // steps is a power of two: the product by its reciprocal is the exact quotient
-                const float delta = __fmul_rn(__fsub_rn(xi.y, xi.x), __frcp_rn((float)g.steps));
-                const float u = JIT ? jit_fraction(g.jitter, jit_ray_key(g.jitter, ro, rd), (int)k, g.steps, j) : 0.5f;
-                const float tj = __fadd_rn(xi.x, __fmul_rn(__fadd_rn((float)j, u), delta));
-#pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                    d[a] = rd[a];
-                    x[a] = __fadd_rn(ro[a], __fmul_rn(tj, rd[a]));
-                }
-                slot = (uint64_t)ray * (uint64_t)g.cap + (uint64_t)(k * (uint32_t)g.steps + (uint32_t)j);
-            }
-            float s_a = 1.0f;  // FP8 only: this row's activation scale for the next MMA
+    if (srv >= 0) {
+        setmaxnreg_dec<kAuxRegs>();
+        if (used) {
+            const int lane_id = threadIdx.x & 31;
+            const uint32_t w_addr = smem_u32(wbuf);
+            // shared-memory descriptors of the first core matrix of W0, W1 and the head; the
+            // start-address field holds address / 16 in 14 bits, and every address here is
+            // below 2^18, so later core matrices are these plus (offset / 16)
+            const uint64_t desc_w0 = sdesc(w_addr + (uint32_t)lay.w0, (uint32_t)K0P * (F8 ? 8u : 16u));
+            const uint64_t desc_wh = sdesc(w_addr + (uint32_t)lay.wh, (uint32_t)lay.kh * (F8 ? 8u : 16u));
+            const uint64_t desc_wo = sdesc(w_addr + (uint32_t)lay.wo, (uint32_t)lay.khead * 16u);
+            const uint64_t desc_bb = sdesc(w_addr + (uint32_t)lay.bb, (uint32_t)kBiasK * 16u);
+            const uint8_t* wall = reinterpret_cast<const uint8_t*>(g.weights);
+            const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
+            uint32_t t_stop = t_end, t_step = 1, t_next;  // the next tile to look up
+            // the looked-up leaf's tile range and crossing range change only at leaf changes
+            uint32_t lk_t0 = 0u, lk_t1 = 0u, lk_x0 = 0u, lk_x1 = 0u;
+            int lk_leaf = -1;
             {
-                constexpr int NX = 3 + 6 * kLX;
-                float f[K0];
-                encode_freq<kLX, 0>(x, f);
-                encode_freq<kLD, NX>(d, f);
-                if constexpr (!F8) {
-                    static_assert(K0P == 96, "layer-0 input is stored in three 32-feature chunks");
-                    store_chunk_perm<0>(a_row, f);
-                    store_chunk_perm<1>(a_row, f);
-                    store_chunk_perm<2>(a_row, f);
+                const uint32_t workers = gridDim.x * (uint32_t)n_groups;
+                const uint32_t wid = blockIdx.x * (uint32_t)n_groups + (uint32_t)gi;
+                if (g.schedule == kSchedInterleaved) {
+                    t_next = g.t_begin + wid;
+                    t_step = workers;
+                } else if (g.schedule == kSchedDynamic) {
+                    t_next = 0u;
+                } else {  // contiguous (also each launch of the per-leaf loop)
+                    const uint32_t span = t_end > g.t_begin ? t_end - g.t_begin : 0u;
+                    const uint32_t per = (span + workers - 1) / workers;
+                    t_next = min(g.t_begin + wid * per, t_end);
+                    t_stop = min(t_next + per, t_end);
+                }
+            }
+            // the stager warp: leaf and crossing ids of tile n (tiles come in increasing order)
+            auto stage_ids = [&](uint32_t n) {
+                if (g.schedule == kSchedDynamic) {
+                    uint32_t v = 0;
+                    if (lane_id == 0) v = atomicAdd(g.tile_counter, 1u) + g.t_begin;
+                    t_next = __shfl_sync(0xffffffffu, v, 0);
+                }
+                uint32_t* dst = id_s + (n & (kIdSlots - 1)) * cpt;
+                const bool any = t_next < t_stop;
+                if (any) {
+                    if (t_next >= lk_t1) {
+                        lk_leaf = leaf_of_tile_warp(g.tile_off, lk_leaf + 1, g.n_leaves, t_next);
+                        lk_t0 = __ldg(g.tile_off + lk_leaf);
+                        lk_t1 = __ldg(g.tile_off + lk_leaf + 1);
+                        lk_x0 = __ldg(g.offsets + lk_leaf);
+                        lk_x1 = __ldg(g.offsets + lk_leaf + 1);
+                    }
+                    for (int c = lane_id; c < cpt; c += 32) {
+                        const uint32_t at = lk_x0 + (t_next - lk_t0) * (uint32_t)cpt + (uint32_t)c;
+                        if (at < lk_x1) cp_async<4>(smem_u32(dst + c), g.order + at);
+                        else dst[c] = 0xffffffffu;
+                    }
                 } else {
-                    static_assert(K0P == 96, "E4M3 layer-0 input is stored as 16 + 8 columns");
-                    float inv = 1.0f;  // static scales: the features as they are
-                    if constexpr (!ST) {  // this row's own scale
-                        float m = 0.0f;
+                    for (int c = lane_id; c < cpt; c += 32) dst[c] = 0xffffffffu;
+                }
+                if (lane_id == 0) leaf_s[n & (kIdSlots - 1)] = any ? lk_leaf : -1;
+                t_next += t_step;
+            };
+            // ... and, its ids staged, the intervals and rays of tile n
+            auto stage_data = [&](uint32_t n) {
+                const uint32_t* ids = id_s + (n & (kIdSlots - 1)) * cpt;
+                const uint32_t dst = smem_u32(data_s + (n & (kDataSlots - 1)) * cpt * 8);
+                for (int c = lane_id; c < cpt; c += 32) {
+                    const uint32_t id = ids[c];
+                    if (id == 0xffffffffu) continue;
+                    const size_t ray = 3 * (size_t)div_maxc(g, id);
+                    cp_async<8>(dst + 32 * c, g.xing + id);
 #pragma unroll
-                        for (int i = 0; i < K0; ++i) m = fmaxf(m, fabsf(f[i]));
-                        inv = m > 0.0f ? 448.0f / m : 0.0f;
-                        s_a = m > 0.0f ? m / 448.0f : 0.0f;
+                    for (int a = 0; a < 3; ++a) {
+                        cp_async<4>(dst + 32 * c + 8 + 4 * a, g.ro + ray + a);
+                        cp_async<4>(dst + 32 * c + 20 + 4 * a, g.rd + ray + a);
                     }
-                    uint32_t w[24];
-#pragma unroll
-                    for (int i = 0; i < 24; ++i) {
-                        // features scaled in pairs; the padding past K0 is zero
-                        float e[4];
-#pragma unroll
-                        for (int u = 0; u < 4; u += 2) {
-                            const int f0 = 4 * i + u;
-                            if (ST) {
-#pragma unroll
-                                for (int q = 0; q < 2; ++q) e[u + q] = f0 + q < K0 ? f[f0 + q < K0 ? f0 + q : 0] : 0.0f;
-                            } else {
-#pragma unroll
-                                for (int q = 0; q < 2; ++q) {
-                                    const int fq = f0 + q;
-                                    e[u + q] = fq < K0 ? f[fq < K0 ? fq : 0] * inv : 0.0f;
-                                }
-                            }
+                }
+            };
+
+            // one phase of bar_s: 32 arrivals when the lanes' copies so far are complete, and one
+            // that releases the plain stores
+            auto publish_stage = [&]() {
+                cp_async_arrive(bar_s);
+                __syncwarp();
+                if (lane_id == 0) mbar_arrive(bar_s);
+            };
+            uint32_t ph_w = 0, ph_h = 0, ph_a = 0;
+            for (uint32_t n = 0; n < 3; ++n) stage_ids(n);
+            __syncwarp();
+            int cur = leaf_s[0];
+            if (cur >= 0 && lane_id == 0)
+                bulk_load(w_addr, wall + (size_t)cur * lay.stride, (uint32_t)lay.stride, bar_w);
+            cp_async_wait_all();
+            __syncwarp();
+            stage_data(0);
+            stage_data(1);
+            publish_stage();
+            bool fresh = true;  // weights loaded but not yet waited for
+            for (uint32_t n = 0;; ++n) {
+                const int leaf = leaf_s[n & (kIdSlots - 1)];
+                if (n > 0) {
+                    // tile n - 1's last epilogue is done (with it this tile's layer-0 input): its
+                    // head, onto the bias in the head columns
+                    if (!wait(bar_a, ph_a)) break;
+                    ph_a ^= 1u;
+                    tc_fence_after();
+                    const uint32_t idd = idesc_bf16(16);
+                    for (int kk = 0; kk < lay.khead / 16; ++kk)
+                        mma_bf16_ts_warp(d_col + kHeadCol, d_col + 8u * kk, desc_wo + 16u * kk, idd, 1u);
+                    mma_commit_warp(bar_h);
+                    if (leaf < 0) break;
+                    // the head reads D, which layer 0 overwrites, and its leaf's weights
+                    if (!wait(bar_h, ph_h)) break;
+                    ph_h ^= 1u;
+                    if (leaf != cur) {  // every row is done with the previous leaf's weights
+                        if (lane_id == 0) {
+                            fence_proxy_async();
+                            bulk_load(w_addr, wall + (size_t)leaf * lay.stride, (uint32_t)lay.stride, bar_w);
                         }
-                        w[i] = pack_e4m3x4(e[0], e[1], e[2], e[3]);
+                        cur = leaf;
+                        fresh = true;
                     }
-                    tmem_st16(a_row, w);
-                    tmem_st8(a_row + 16u, w + 16);
+                } else if (leaf < 0) {
+                    break;
                 }
-            }
-            tmem_st_wait();
-            tc_fence_before();
-            wg_bar(bar_id);
-            if (pending) {
-                // on expiry the leader issues no more MMAs, so the group's next wait runs
-                // out too and the whole group leaves through it
-                if (leader_warp) {
-                    const bool okw = mbar_wait_bounded(bar_m, ph_m);
-                    if (!__all_sync(0xffffffffu, okw)) head_bad = true;
+                if (fresh) {
+                    if (!wait(bar_w, ph_w)) break;
+                    ph_w ^= 1u;
+                    fresh = false;
                 }
-                ph_m ^= 1u;
-                pending = false;
-            }
-
-            int leaf_n = leaf;
-            uint32_t id_n = 0xffffffffu;
-            uint32_t t_next = t_stop;
-
-            // ---- hidden layers; the last epilogue issues the head MMA
-            int kin = K0P;
+                int kin = K0P;
 #pragma unroll
-            for (int l = 0; l < hidden; ++l) {
-                if (!ok) break;
-                if (leader_warp && !head_bad) {
+                for (int l = 0; l < hidden; ++l) {
+                    if (l > 0 || n == 0) {
+                        if (!wait(bar_a, ph_a)) break;
+                        ph_a ^= 1u;
+                    }
                     tc_fence_after();
                     // this layer's first weight core matrix, then 256 B (16 descriptor
                     // units) per K step
@@ -459,72 +489,301 @@ __global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n
                         if constexpr (ST)
                             mma_bf16_ts_warp(d_col, a_col + (uint32_t)(kOnesStep / 2),
                                              desc_bb + (uint64_t)(((size_t)l * W * kBiasK * 2) >> 4), idesc_bf16(W), 0u);
+                        const uint32_t a8 = a_col + (l == 0 ? kA0Col8 : 0u);
                         for (int kk = 0; kk < kin / KI; ++kk)
-                            mma_e4m3_ts_warp(d_col, a_col + 8u * kk, b_desc + 16u * kk, idd, (ST || kk > 0) ? 1u : 0u);
+                            mma_e4m3_ts_warp(d_col, a8 + 8u * kk, b_desc + 16u * kk, idd, (ST || kk > 0) ? 1u : 0u);
                     } else {
                         const uint32_t idd = idesc_bf16(W);
                         // layer 0 starts from zero (its bias is folded in); a later layer
                         // first writes its bias (the constant-1 input columns against the
-                        // layer's bias operand), then accumulates onto it
+                        // layer's bias operand), then accumulates onto it; its input's
+                        // features 32..63 sit in the head columns
                         if (l > 0)
                             mma_bf16_ts_warp(d_col, a_col + (uint32_t)(kOnesStep / 2),
                                              desc_bb + (uint64_t)(((size_t)(l - 1) * W * kBiasK * 2) >> 4), idd, 0u);
                         for (int kk = 0; kk < kin / KI; ++kk)
-                            mma_bf16_ts_warp(d_col, a_col + 8u * kk, b_desc + 16u * kk, idd,
-                                             (kk > 0 || l > 0) ? 1u : 0u);
+                            mma_bf16_ts_warp(d_col,
+                                             l > 0 && kk > 1 ? d_col + kHeadCol + 8u * (kk - 2) : a_col + 8u * kk,
+                                             b_desc + 16u * kk, idd, (kk > 0 || l > 0) ? 1u : 0u);
                     }
                     mma_commit_warp(bar_m);
-                }
-                // next tile of this worker, its leaf and this row's crossing id
-                auto next_lookup = [&](uint32_t tn) {
-                    t_next = tn;
-                    if (t_next < t_stop) {
-                        if (t_next >= lk_t1 || t_next < lk_t0) {  // another leaf (rare)
-                            if (t_next - t <= 8u && t_next >= lk_t1) {
-                                while (__ldg(g.tile_off + leaf_n + 1) <= t_next) ++leaf_n;
-                            } else {
-                                leaf_n = leaf_of_tile(g.tile_off, g.n_leaves, t_next);
-                            }
-                            leaf_ranges(leaf_n);
-                        }
-                        const uint32_t c = lk_x0 + (t_next - lk_t0) * (uint32_t)(kTileRows >> g.lg_steps) + (uint32_t)ci;
-                        id_n = c < lk_x1 ? __ldg(g.order + c) : 0xffffffffu;
+                    kin = lay.kh;
+                    // behind the later layers' issue, where the compute warps are in their
+                    // epilogues: the slots' previous contents were read before tile n - 1's
+                    // last layer, and tile n + 2's ids were copied a tile ago
+                    if (l == (hidden > 1 ? 1 : 0)) {
+                        cp_async_wait_all();
+                        __syncwarp();
+                        stage_data(n + 2);
+                        publish_stage();
                     }
-                };
-                const bool dyn = g.schedule == kSchedDynamic;
-                if (l == 0 && dyn && leader) sh->next_tile[grp] = atomicAdd(g.tile_counter, 1u) + g.t_begin;
-                // The next tile's dependent loads are spread over the layers, each issued
-                // while MMAs run and consumed a layer later: static schedules know the next
-                // tile already, so its leaf and crossing id are looked up before the layer-0
-                // wait; its interval and ray at layer l_xd; the previous tile's outputs are
-                // stored at layer l_sh.
-                const int l_xd = hidden > 1 ? 1 : 0;
-                const int l_sh = hidden > 3 ? 3 : hidden - 1;
-                if (!dyn && l == 0) next_lookup(t + t_step);
-                if (!dyn && l > 0 && l == l_xd) crossing_data(g, id_n, xi, ro, rd);
-                if (zpend && l == l_sh) store_head();
-                // Every thread waits for the MMAs itself (the dynamic schedule's first
-                // layer keeps the group barrier, which publishes the next tile).  A thread
-                // whose wait ran out carries that to the group's next barrier, where the
-                // whole group learns of it and leaves together.
-                bool late = false;
-                if (dyn && l == 0) ok = group_wait(bar_m, ph_m, bar_id, flag, leader);
-                else late = !mbar_wait_bounded(bar_m, ph_m);
-                ph_m ^= 1u;
+                    if (l == (hidden > 2 ? 2 : hidden - 1)) stage_ids(n + 3);
+                }
                 if (!ok) break;
+            }
+            cp_async_wait_all();  // none in flight when the CTA ends
+            if (!ok && lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
+        }
+    } else {
+        setmaxnreg_inc<kComputeRegs>();
+        const uint32_t lane = (uint32_t)(32 * q) << 16;
+        const uint32_t d_row = d_col + lane;  // this warp's lanes
+        const uint32_t a_row = a_col + lane;
+        const float* bias = reinterpret_cast<const float*>(wbuf + lay.bias);
+        if constexpr (F8 && ST) {
+            // the BF16 constant-1 input columns of the bias MMAs (the K = 16 step at
+            // A columns 40..47, ones at its columns 10..12), which no E4M3 operand
+            // reaches: written once
+            const uint32_t c8[8] = {0u, 0u, 0u, 0u, 0u, pack_bf16(1.0f, 1.0f), pack_bf16(1.0f, 0.0f), 0u};
+            static_assert((kOnesCol - kOnesStep) / 2 == 5, "ones at K-step columns 10..12");
+            tmem_st8(a_row + (uint32_t)(kOnesStep / 2), c8);
+        }
+
+        const int ci = tig >> g.lg_steps;              // crossing of this row within a tile
+        const int j = tig - (ci << g.lg_steps);        // sample of this row within its crossing
+        // the layer's input (or the tile's last accumulator row) is written: one arrival per warp
+        auto publish = [&]() {
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if ((threadIdx.x & 31) == 0) mbar_arrive(bar_a);
+        };
+        uint32_t id_prev = 0xffffffffu;  // the crossing whose head result waits
+        uint32_t zr[4] = {0u, 0u, 0u, 0u};
+        auto store_head = [&]() {
+            if (id_prev != 0xffffffffu) {  // 4 x FP16; sigma saturates at the FP16 maximum
+                const uint32_t ray = div_maxc(g, id_prev);
+                const uint32_t k = id_prev - ray * (uint32_t)g.maxc;
+                // 64-bit: rays * cap may exceed 2^32
+                const uint64_t slot_prev = (uint64_t)ray * (uint64_t)g.cap + (uint64_t)((k << g.lg_steps) + (uint32_t)j);
+                uint2 o;
+                o.x = pack_f16(fminf(softplus_f(__uint_as_float(zr[0])), 65504.0f), sigmoid_f(__uint_as_float(zr[1])));
+                o.y = pack_f16(sigmoid_f(__uint_as_float(zr[2])), sigmoid_f(__uint_as_float(zr[3])));
+                static_cast<uint2*>(g.slot_out)[slot_prev] = o;
+            }
+        };
+        // this row's sample of the tile to be encoded: its crossing, position and direction
+        uint32_t id = 0xffffffffu;
+        float rd[3] = {0.f, 0.f, 0.f};
+        float x[3];  // its position
+        auto place_sample = [&](uint32_t n) {
+            id = id_s[(n & (kIdSlots - 1)) * cpt + ci];
+            const float4* p = reinterpret_cast<const float4*>(data_s + ((n & (kDataSlots - 1)) * cpt + ci) * 8);
+            const float4 u0 = p[0], u1 = p[1];
+            if (id != 0xffffffffu) {
+                const float ro[3] = {u0.z, u0.w, u1.x};
+                rd[0] = u1.y;
+                rd[1] = u1.z;
+                rd[2] = u1.w;
+                // steps is a power of two: the product by its reciprocal is the exact quotient
+                const float delta = __fmul_rn(__fsub_rn(u0.y, u0.x), __frcp_rn((float)g.steps));
+                float u = 0.5f;
+                if constexpr (JIT) {
+                    const uint32_t k = id - div_maxc(g, id) * (uint32_t)g.maxc;
+                    u = jit_fraction(g.jitter, jit_ray_key(g.jitter, ro, rd), (int)k, g.steps, j);
+                }
+                const float tj = __fadd_rn(u0.x, __fmul_rn(__fadd_rn((float)j, u), delta));
+#pragma unroll
+                for (int a = 0; a < 3; ++a) x[a] = __fadd_rn(ro[a], __fmul_rn(tj, rd[a]));
+            } else {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) x[a] = rd[a] = 0.f;
+            }
+        };
+
+        // ---- the layer-0 input of the sample in three parts (kperm's column order for BF16,
+        // the canonical one for E4M3), each computed under one layer's MMAs and stored where
+        // its columns are free:
+        //   part D   gamma(d)            (static and BF16; from the anchor at octave 0)
+        //   part H   x's octaves 5-9     (anchor at octave 5)
+        //   part L   x and its octaves 0-4
+        // BF16: D = words 17..23 and 39..44 and d.x (high half of word 16), H = words 24..38,
+        // L = words 0..15 and the low half of word 16, words 45..47 constant.
+        // E4M3, static: D = words 16..23 and feature 63, H = words 9..15 and features 33..35,
+        // L = words 0..7 and feature 32 (word 8).
+        // E4M3, per-row scales: the row's maximum needs every feature: all under one layer.
+        constexpr int NPD = 7, NPK = F8 ? 1 : 6, NPH = !F8 ? 16 : (ST ? 8 : 24), NPL = F8 ? 9 : 17;
+        uint32_t pk6[NPK];         // BF16: words 39..44, kept until parts H and L are stored
+        float dx = 0.f, h3[3] = {0.f, 0.f, 0.f};
+        float s_n = 1.0f;          // per-row scales: the encoded row's activation scale
+        // pd: BF16 words 17..23; E4M3 words 16..22
+        auto encode_d = [&](uint32_t (&pd)[NPD]) {
+            if constexpr (!F8) {
+                float f[24];
+                encode_octaves<0, 4, 0>(rd, f);
+                dx = rd[0];
+                pd[0] = pack_bf16(rd[1], rd[2]);
+#pragma unroll
+                for (int i = 0; i < 6; ++i) {
+                    pd[1 + i] = pack_bf16(f[2 * i], f[2 * i + 1]);
+                    pk6[i] = pack_bf16(f[12 + 2 * i], f[13 + 2 * i]);
+                }
+                pin(pd);
+                pin(pk6);
+            } else if constexpr (ST) {
+                float f[28];  // features 63 .. 90
+#pragma unroll
+                for (int a = 0; a < 3; ++a) f[a] = rd[a];
+                encode_octaves<0, 4, 3>(rd, f);
+                f[27] = 0.0f;
+                dx = f[0];
+#pragma unroll
+                for (int i = 0; i < 6; ++i)
+                    pd[i] = pack_e4m3x4(f[4 * i + 1], f[4 * i + 2], f[4 * i + 3], f[4 * i + 4]);
+                pd[6] = pack_e4m3x4(f[25], f[26], 0.0f, 0.0f);
+                pin(pd);
+            }
+        };
+        // part D into the columns free after layer 0 (BF16: column 16 is completed by part L)
+        auto store_d = [&](const uint32_t (&pd)[NPD]) {
+            if constexpr (!F8) {
+                const uint32_t w[8] = {0u, pd[0], pd[1], pd[2], pd[3], pd[4], pd[5], pd[6]};
+                tmem_st8(a_row + 16u, w);
+            } else if constexpr (ST) {
+                const uint32_t w[8] = {pd[0], pd[1], pd[2], pd[3], pd[4], pd[5], pd[6], 0u};
+                tmem_st8(a_row + kA0Col8 + 16u, w);
+            }
+        };
+        // ph: part H (per-row scales: the whole row)
+        auto encode_h = [&](uint32_t (&ph)[NPH]) {
+            if constexpr (F8 && !ST) {
+                float f[K0];
+                encode_freq<kLX, 0>(x, f);
+                encode_freq<kLD, 3 + 6 * kLX>(rd, f);
+                float m = 0.0f;
+#pragma unroll
+                for (int i = 0; i < K0; ++i) m = fmaxf(m, fabsf(f[i]));
+                const float inv = m > 0.0f ? 448.0f / m : 0.0f;
+                s_n = m > 0.0f ? m / 448.0f : 0.0f;
+#pragma unroll
+                for (int i = 0; i < 24; ++i) {
+                    float e[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) e[u] = 4 * i + u < K0 ? f[4 * i + u < K0 ? 4 * i + u : 0] * inv : 0.0f;
+                    ph[i] = pack_e4m3x4(e[0], e[1], e[2], e[3]);
+                }
+                pin(ph);
+            } else {
+                float f[30];
+                encode_octaves<5, 10, 0>(x, f);
+                if constexpr (!F8) {
+#pragma unroll
+                    for (int i = 0; i < 15; ++i) ph[i] = pack_bf16(f[2 * i], f[2 * i + 1]);
+                    ph[15] = pk6[0];
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 3; ++a) h3[a] = f[a];
+                    ph[0] = 0u;
+#pragma unroll
+                    for (int i = 0; i < 6; ++i)
+                        ph[1 + i] = pack_e4m3x4(f[4 * i + 3], f[4 * i + 4], f[4 * i + 5], f[4 * i + 6]);
+                    ph[7] = pack_e4m3x4(f[27], f[28], f[29], dx);
+                }
+                pin(ph);
+            }
+        };
+        auto store_h = [&](const uint32_t (&ph)[NPH]) {
+            if constexpr (!F8) {
+                tmem_st16(a_row + 24u, ph);
+            } else if constexpr (ST) {
+                tmem_st8(a_row + kA0Col8 + 8u, ph);
+            } else {
+                tmem_st16(a_row + kA0Col8, ph);
+                tmem_st8(a_row + kA0Col8 + 16u, ph + 16);
+            }
+        };
+        auto encode_l = [&](uint32_t (&pl)[NPL]) {
+            if constexpr (!(F8 && !ST)) {
+                float f[36];
+#pragma unroll
+                for (int a = 0; a < 3; ++a) f[a] = x[a];
+                encode_octaves<0, 5, 3>(x, f);
+                if constexpr (!F8) {
+#pragma unroll
+                    for (int i = 0; i < 16; ++i) pl[i] = pack_bf16(f[2 * i], f[2 * i + 1]);
+                    pl[16] = pack_bf16(f[32], dx);
+                } else {
+#pragma unroll
+                    for (int i = 0; i < 8; ++i)
+                        pl[i] = pack_e4m3x4(f[4 * i], f[4 * i + 1], f[4 * i + 2], f[4 * i + 3]);
+                    pl[8] = pack_e4m3x4(f[32], h3[0], h3[1], h3[2]);
+                }
+                pin(pl);
+            }
+        };
+        // part L and what waited for the last layer's completion (BF16: the K step with the
+        // constant ones, columns 40..47)
+        auto store_l = [&](const uint32_t (&pl)[NPL]) {
+            if constexpr (!F8) {
+                tmem_st16(a_row, pl);
+                tmem_st1(a_row + 16u, pl[16]);
+                const uint32_t w[8] = {pk6[1], pk6[2], pk6[3], pk6[4], pk6[5], pack_bf16(1.0f, 1.0f),
+                                       pack_bf16(1.0f, 0.0f), 0u};
+                tmem_st8(a_row + 40u, w);
+            } else if constexpr (ST) {
+                tmem_st8(a_row + kA0Col8, pl);
+                tmem_st1(a_row + kA0Col8 + 8u, pl[8]);
+            }
+        };
+
+        // ---- the first tile's input
+        uint32_t id_cur = 0xffffffffu;  // this row's crossing of the current tile
+        float s_a = 1.0f;  // per-row scales: this row's activation scale for the next MMA
+        if (wait(bar_s, 0u) && leaf_s[0] >= 0) {
+            place_sample(0);
+            id_cur = id;
+            uint32_t pd[NPD], ph[NPH], pl[NPL];
+            encode_d(pd);
+            store_d(pd);
+            encode_h(ph);
+            store_h(ph);
+            encode_l(pl);
+            tmem_st_wait();  // part L completes a column of part D (BF16) or H (E4M3)
+            store_l(pl);
+            s_a = s_n;
+            publish();
+        }
+        uint32_t ph_m = 0, ph_w = 0, n = 0;
+        int cur = -1;
+        for (; ok; ++n) {
+            const int leaf = leaf_s[n & (kIdSlots - 1)];
+            if (leaf < 0) break;
+            if (leaf != cur) {  // its weights' biases and scales are read below
+                if (!wait(bar_w, ph_w)) break;
+                ph_w ^= 1u;
+                cur = leaf;
+            }
+#pragma unroll
+            for (int l = 0; l < hidden; ++l) {
+                const bool last = l + 1 == hidden;
+                // ---- work that overlaps this layer's MMAs: the next tile's sample is placed and
+                // its direction encoded, then its position; the previous tile's outputs are
+                // stored under layer 2
+                const int l_h = hidden > 1 ? 1 : 0;
+                const int l_sh = hidden > 2 ? 2 : hidden - 1;
+                uint32_t pd[NPD], ph[NPH], pl[NPL];
+                if (l == 0) {
+                    if (n > 0 && !wait(bar_s, n & 1u)) break;
+                    place_sample(n + 1);
+                    encode_d(pd);
+                }
+                if (l == l_h) {
+                    encode_h(ph);
+                    if (l > 0) store_h(ph);  // layer 0 has completed
+                }
+                if (n > 0 && l == l_sh && l > 0) store_head();
+                if (last) encode_l(pl);
+                if (!wait(bar_m, ph_m)) break;
+                ph_m ^= 1u;
                 tc_fence_after();
-                if (dyn && l == 0) next_lookup(sh->next_tile[grp]);  // published by the wait's barrier
-                if ((dyn || l_xd == 0) && l == l_xd) crossing_data(g, id_n, xi, ro, rd);
+                if (l == 0) {
+                    store_d(pd);
+                    if (l_h == 0) store_h(ph);
+                }
                 const float* b = bias + (size_t)l * W;
                 const float* sw = reinterpret_cast<const float*>(wbuf + lay.sw) + (size_t)l * W;
-                const bool last = l + 1 == hidden;
                 // the previous tile's head result: loaded now, waited for with D below
-                if (l == 0 && have_out) {
-                    tmem_ld4_nowait(d_row + kHeadCol, zr);
-                    slot_z = slot_prev;
-                    have_out = false;
-                    zpend = true;
-                }
+                if (l == 0 && n > 0) tmem_ld4_nowait(d_row + kHeadCol, zr);
                 // pre-activation of 4 consecutive columns c0..c0+3 of this row
                 auto pre4 = [&](const float* v, int c0, float2& p01, float2& p23) {
                     if constexpr (F8 && !ST) {
@@ -541,21 +800,7 @@ __global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n
                 };
                 if (!last) {
                     if constexpr (!F8) {
-                        float vr[W];
-                        tmem_ld_row<W>(d_row, vr);
-#pragma unroll
-                        for (int h = 0; h < W / 32; ++h) {
-                            const float* v = vr + 32 * h;
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                float2 p01, p23;
-                                pre4(v + 4 * c, 32 * h + 4 * c, p01, p23);
-                                pk[2 * c + 0] = pack_relu_bf16(p01.x, p01.y);
-                                pk[2 * c + 1] = pack_relu_bf16(p23.x, p23.y);
-                            }
-                            tmem_st16(a_row + 16u * h, pk);
-                        }
+                        relu_row<W>(d_row, a_row, d_row + kHeadCol);
                     } else if constexpr (ST) {
                         // relu(acc) is the next layer's E4M3 input (its channel scales are
                         // this layer's output-channel scales, folded into the next weights)
@@ -596,31 +841,19 @@ __global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n
                         if constexpr (W / 4 == 16) tmem_st16(a_row, pk);
                         else tmem_st8(a_row, pk);
                     }
-                    tmem_st_wait();
-                    tc_fence_before();
-                    if (wg_bar_any(bar_id, late)) {
-                        ok = false;
-                        break;
-                    }
-                    kin = lay.kh;
+                    publish();
                 } else {
                     // relu(h) as BF16 into this group's D columns (each 32-column block is
-                    // read before it is overwritten), the head bias into D columns
+                    // read before it is overwritten), the head bias into columns
                     // kHeadCol..+3, then the head MMA (16 x khead) accumulates onto it
                     if constexpr (!F8) {
-                        float vr[W];
-                        tmem_ld_row<W>(d_row, vr);
-#pragma unroll
-                        for (int h = 0; h < W / 32; ++h) {
-                            const float* v = vr + 32 * h;
-                            uint32_t pk[16];
-#pragma unroll
-                            for (int c = 0; c < 8; ++c) {
-                                pk[2 * c + 0] = pack_relu_bf16(v[4 * c + 0], v[4 * c + 1]);
-                                pk[2 * c + 1] = pack_relu_bf16(v[4 * c + 2], v[4 * c + 3]);
-                            }
-                            tmem_st16(d_row + 16u * h, pk);
-                        }
+                        if (l == 0) tmem_st_wait();  // part L completes a column of part D
+                        store_l(pl);
+                        relu_row<W>(d_row, d_row, d_row + 16u);
+                    } else if constexpr (ST) {
+                        if (l <= 1) tmem_st_wait();  // part L completes a column of part H
+                        store_l(pl);
+                        relu_row<W>(d_row, d_row, d_row + 16u);
                     } else {  // E4M3: per-row scales need the channel scales and the bias
 #pragma unroll
                         for (int h = 0; h < W / 32; ++h) {
@@ -636,40 +869,24 @@ __global__ void __launch_bounds__(128 * kMaxGroups, 1) k_mlp_tc(MlpArgs g, int n
                             }
                             tmem_st16(d_row + 16u * h, pk);
                         }
+                        s_a = s_n;  // the next tile's encoded row
                     }
+                    if (l == 0 && n > 0) tmem_ld_wait_regs(zr);  // one hidden layer: read before the bias is written
                     tmem_st4(d_row + kHeadCol, bias + (size_t)hidden * W);
-                    tmem_st_wait();
-                    tc_fence_before();
-                    if (wg_bar_any(bar_id, late)) {
-                        ok = false;
-                        break;
-                    }
-                    if (leader_warp) {
-                        tc_fence_after();
-                        const uint32_t idd = idesc_bf16(16);
-                        for (int kk = 0; kk < lay.khead / 16; ++kk)
-                            mma_bf16_ts_warp(d_col + kHeadCol, d_col + 8u * kk, desc_wo + 16u * kk, idd, 1u);
-                        mma_commit_warp(bar_m);
-                    }
-                    pending = true;
-                    have_out = true;
-                    slot_prev = slot;
+                    publish();
+                    if (l == 0 && n > 0) store_head();  // one hidden layer
+                    id_prev = id_cur;
                 }
             }
-            if (zpend) store_head();  // one hidden layer: stored after the head MMA issue
-            leaf = leaf_n;
-            id = id_n;
-            t = t_next;
+            id_cur = id;
         }
-        if (ok && pending) ok = head_group_wait();
-        if (ok && have_out) {
+        if (ok && n > 0 && wait(bar_h, (n - 1u) & 1u)) {  // the last tile's head
             tc_fence_after();
             tmem_ld4_nowait(d_row + kHeadCol, zr);
-            tmem_ld_wait();
-            slot_z = slot_prev;
+            tmem_ld_wait_regs(zr);
             store_head();
         }
-        if (!ok && leader) atomicCAS(g.err, 0, kDevErrTimeout);
+        if (!ok && (threadIdx.x & 31) == 0) atomicCAS(g.err, 0, kDevErrTimeout);
     }
     tc_fence_before();
     __syncthreads();
@@ -1036,11 +1253,13 @@ __global__ void k_wait_selftest(unsigned long long limit, int* err) {
     if (threadIdx.x == 0 && !mbar_wait_bounded(smem_u32(&bar), 0, limit)) atomicCAS(err, 0, kDevErrTimeout);
 }
 
+// Groups whose weights and staged crossings fit the shared memory (cpt crossings per tile;
+// 16 at 8 samples per crossing).
 template <int W, bool F8>
-int max_groups_for(int hidden, int max_smem) {
+int max_groups_for(int hidden, int max_smem, int cpt = 16) {
     constexpr int K0 = (3 + 6 * kLX) + (3 + 6 * kLD);
     const TcLayout lay(W, hidden, K0, F8);
-    int groups = (int)((max_smem - (int)sizeof(TcShared) - 64) / (int)lay.stride);
+    int groups = (int)((max_smem - (int)sizeof(TcShared) - 64) / (int)(lay.stride + stage_bytes(cpt)));
     return groups > kMaxGroups ? kMaxGroups : groups;
 }
 
@@ -1120,16 +1339,21 @@ cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid) {
     int dev = 0, max_smem = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-    const int groups = a.groups;
-    if (groups < 1 || groups > max_groups_for<W, F8>(a.hidden, max_smem)) return cudaErrorInvalidConfiguration;
+    const int cpt = kTileRows >> a.lg_steps;
+    if (a.groups < 1 || a.groups > max_groups_for<W, F8>(a.hidden, max_smem)) return cudaErrorInvalidConfiguration;
+    // fewer samples per crossing stage more crossings per tile: a large network may then
+    // fit one group less
+    const int fit = max_groups_for<W, F8>(a.hidden, max_smem, cpt);
+    const int groups = a.groups < fit ? a.groups : fit;
+    if (groups < 1) return cudaErrorInvalidConfiguration;
     const uint32_t cols = 512;  // kGroupCols per group: the whole TMEM, so one CTA per SM
     // at least half of the SM's shared memory, so that a second CTA can never become
     // resident on the SM and wait in tcgen05.alloc for columns this CTA holds
-    size_t smem = lay.stride * groups + sizeof(TcShared) + 64;
+    size_t smem = (lay.stride + stage_bytes(cpt)) * groups + sizeof(TcShared) + 64;
     if (smem < (size_t)max_smem / 2 + 1024) smem = (size_t)max_smem / 2 + 1024;
     const bool hc = a.hidden == kHiddenFor<W>;
     const bool st = F8 && a.act_static;
-#define AMNERF_TC(ST_, HC_, J_) k_mlp_tc<W, F8, ST_, HC_, J_><<<grid, 128 * groups, smem, s>>>(a, groups, cols)
+#define AMNERF_TC(ST_, HC_, J_) k_mlp_tc<W, F8, ST_, HC_, J_><<<grid, 128 * (groups + 1), smem, s>>>(a, groups, cols)
     if (a.jitter) {
         if (st) { if (hc) AMNERF_TC(F8, kHiddenFor<W>, true); else AMNERF_TC(F8, 0, true); }
         else { if (hc) AMNERF_TC(false, kHiddenFor<W>, true); else AMNERF_TC(false, 0, true); }
@@ -1204,7 +1428,7 @@ void pack_tc_leaf(const float* src, uint8_t* dst, int width, int hidden, int k0,
                     sc = m > 0.0f ? m / 448.0f : 1.0f;
                 }
                 s_out[n] = sc;
-                sw[(size_t)l * width + n] = sc;
+                if (!stat) sw[(size_t)l * width + n] = sc;
                 for (int k = 0; k < kin; ++k) base[cm_offset8(n, k, K)] = f2e4m3(row[k] * alpha[k] / sc);
                 bias[(size_t)l * width + n] = stat ? bl[n] / sc : bl[n];
                 if (stat) put_bias_operand(l, n, bl[n] / sc);

@@ -40,6 +40,20 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
 }
 
+__device__ __forceinline__ void mbar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+// Registers per thread of this warpgroup from here on (all of its warps execute it).
+template <int R>
+__device__ __forceinline__ void setmaxnreg_inc() {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(R));
+}
+template <int R>
+__device__ __forceinline__ void setmaxnreg_dec() {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(R));
+}
+
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t phase) {
     uint32_t ok;
     asm volatile(
@@ -63,20 +77,6 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint32_t bar, uint32_t phase,
 
 __device__ __forceinline__ void wg_bar(int id) { asm volatile("barrier.sync %0, 128;" ::"r"(id) : "memory"); }
 
-// The group's named barrier (128 threads) that also ORs a flag over the group: every
-// thread leaves with the same answer, so a group that learns of a failed wait here
-// leaves its loop together (no thread is left waiting at a later barrier).
-__device__ __forceinline__ bool wg_bar_any(int id, bool v) {
-    uint32_t r;
-    asm volatile(
-        "{\n\t.reg .pred pi, po;\n\tsetp.ne.u32 pi, %2, 0;\n\tbarrier.cta.red.or.pred po, %1, 128, pi;\n\t"
-        "selp.u32 %0, 1, 0, po;\n\t}"
-        : "=r"(r)
-        : "r"(id), "r"(v ? 1u : 0u)
-        : "memory");
-    return r != 0;
-}
-
 // One thread of the group (its leader) polls the mbarrier (bounded) while the other
 // 127 sleep at the group's named barrier, so waiting groups take no issue slots from
 // working ones.  The flag carries the outcome to the whole group.
@@ -96,6 +96,19 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                  "l"(src), "r"(bytes), "r"(bar)
                  : "memory");
 }
+
+// An asynchronous copy of N (4 or 8) bytes from global to shared memory, and the wait for
+// all of this thread's.
+template <int N>
+__device__ __forceinline__ void cp_async(uint32_t dst, const void* src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(src), "n"(N) : "memory");
+}
+// One arrival on an mbarrier (counted in its initial count) once all of this thread's
+// asynchronous copies so far are complete.
+__device__ __forceinline__ void cp_async_arrive(uint32_t bar) {
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // Shared-memory matrix descriptor: K-major, no swizzle, LBO = 128 B, SBO = sbo bytes.
 __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t sbo) {
@@ -163,6 +176,10 @@ __device__ __forceinline__ void tmem_st4(uint32_t taddr, const float* v) {
     asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(taddr), "r"(__float_as_uint(v[0])),
                  "r"(__float_as_uint(v[1])), "r"(__float_as_uint(v[2])), "r"(__float_as_uint(v[3]))
                  : "memory");
+}
+
+__device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t w) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x1.b32 [%0], {%1};" ::"r"(taddr), "r"(w) : "memory");
 }
 
 // The N FP32 values at shared address b (the same for every row) into columns [0, N)
@@ -235,6 +252,12 @@ __device__ __forceinline__ void tmem_ld32_nowait(uint32_t taddr, uint32_t* r) {
 }
 
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// The wait for a load of 4 columns, tied to its registers, so that no use of them can be
+// moved in front of it.
+__device__ __forceinline__ void tmem_ld_wait_regs(uint32_t (&r)[4]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3])::"memory");
+}
 
 // 32 consecutive FP32 columns of this thread's TMEM lane (load + wait; the E4M3
 // epilogues, whose register budget is tighter, read a row in two halves).
@@ -318,6 +341,21 @@ __device__ __forceinline__ int leaf_of_tile(const uint32_t* __restrict__ tile_of
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
         if (__ldg(tile_off + mid) <= t) lo = mid; else hi = mid;
+    }
+    return lo;
+}
+
+// The same by a whole converged warp, with the leaf known to be in [lo, hi): each step's 32
+// pivots are loaded at once, so 8192 networks take three dependent loads instead of 13.
+__device__ __forceinline__ int leaf_of_tile_warp(const uint32_t* __restrict__ tile_off, int lo, int hi, uint32_t t) {
+    const int lane = threadIdx.x & 31;
+    while (hi - lo > 1) {  // tile_off[lo] <= t < tile_off[hi]
+        const int step = (hi - lo + 31) >> 5;
+        const int i = lo + step * lane;
+        const bool le = i < hi && __ldg(tile_off + i) <= t;  // lane 0: true
+        const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
+        lo += step * k;
+        hi = min(hi, lo + step);
     }
     return lo;
 }
@@ -424,22 +462,6 @@ __host__ __device__ constexpr int kperm(int k) {
 }
 constexpr int kOnesStep = 80;  // first column of the K = 16 step that holds the constant-1 columns
 constexpr int kOnesCol = 90;   // the constant-1 columns are kOnesCol .. kOnesCol + 2
-
-// Columns [32 C, 32 C + 32) of the layer-0 input in kperm order, from the canonical
-// features f, packed two per word and written to this thread's TMEM lane.
-template <int C, int N>
-__device__ __forceinline__ void store_chunk_perm(uint32_t a_row, const float (&f)[N]) {
-    uint32_t w[16];
-#pragma unroll
-    for (int i = 0; i < 16; ++i) {
-        const int k0 = 32 * C + 2 * i, k1 = k0 + 1;
-        const int c0 = kperm(k0), c1 = kperm(k1);
-        const float v0 = c0 >= 0 ? f[c0 >= 0 ? c0 : 0] : (c0 == -2 ? 0.0f : 1.0f);
-        const float v1 = c1 >= 0 ? f[c1 >= 0 ? c1 : 0] : (c1 == -2 ? 0.0f : 1.0f);
-        w[i] = pack_bf16(v0, v1);
-    }
-    tmem_st16(a_row + 16u * C, w);
-}
 
 // Features [32 c, 32 c + 32) of f packed two per word (even feature in the low half)
 // and written to this thread's TMEM lane at A column 16 c; feature N (one past the

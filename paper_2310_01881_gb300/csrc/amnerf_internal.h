@@ -154,6 +154,15 @@ struct MlpArgs {
 };
 cudaError_t launch_mlp_simt(cudaStream_t s, const MlpArgs& a, int grid);
 cudaError_t launch_mlp_tc(cudaStream_t s, const MlpArgs& a, int grid, int prec);
+// FP32 networks on the tensor cores (k_mlp_split.cu): bytes of a network's split weights (0:
+// the encoding or width has no such path), whether they fit beside `steps` samples per
+// crossing, kernel attributes, the split weights of n_nets networks from the SIMT blob.
+size_t split_leaf_stride_bytes(int width, int hidden, int lx, int ld);
+bool split_fits(int width, int hidden, int steps);
+cudaError_t prepare_mlp_split(int width);
+cudaError_t launch_split_pack(cudaStream_t s, const float* simt, size_t simt_stride, int n_nets, int width, int hidden,
+                              void* out);
+cudaError_t launch_mlp_split(cudaStream_t s, const MlpArgs& a, int grid);
 // Kernel attributes (dynamic shared memory) and the largest group count the tcgen05
 // kernel supports for this shape; called at weight-load time, outside any capture.
 cudaError_t prepare_mlp_tc(int width, int hidden, int k0, int prec, int* max_groups);

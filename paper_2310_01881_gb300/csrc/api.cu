@@ -39,6 +39,7 @@ struct amnerf_ctx {
     int k0 = 0;
     size_t leaf_stride = 0;  // bytes
     void* d_weights = nullptr;
+    void* d_split = nullptr;  // FP32 networks: their split operands (tensor-core path; null: SIMT only)
     // per-network scratch (sized for kMaxNets)
     uint32_t* d_counts = nullptr;
     uint32_t* d_offsets = nullptr;
@@ -312,6 +313,7 @@ void amnerf_destroy(amnerf_ctx* ctx) {
     dfree(ctx->d_walk);
     dfree(ctx->d_grid);
     dfree(ctx->d_weights);
+    dfree(ctx->d_split);
     dfree(ctx->d_amax);
     dfree(ctx->d_counts);
     dfree(ctx->d_offsets);
@@ -394,6 +396,7 @@ amnerf_status amnerf_build_tree(amnerf_ctx* ctx, const float* grid_host, int G, 
     ctx->tree_depth = depth;
     ctx->mlp_loaded = false;
     dfree(ctx->d_weights);
+    dfree(ctx->d_split);
     if (n_leaves_out) *n_leaves_out = nl;
     return AMNERF_OK;
 }
@@ -449,9 +452,28 @@ static amnerf_status load_impl(amnerf_ctx* ctx, const amnerf_mlp_desc* desc, int
     }
     if (ctx->stream) cudaStreamSynchronize(ctx->stream);
     dfree(ctx->d_weights);
+    dfree(ctx->d_split);
     ctx->mlp_loaded = false;
     CK(cudaMalloc(&ctx->d_weights, blob.size()), "weight allocation");
     CK(cudaMemcpy(ctx->d_weights, blob.data(), blob.size(), cudaMemcpyHostToDevice), "weight upload");
+    if (m.prec == AMNERF_FP32) {
+        // the same networks as split operands (k_mlp_split.cu), packed on the device from the
+        // blob just uploaded; without them (shape, shared memory or device memory) the SIMT
+        // kernel renders
+        const size_t split = split_leaf_stride_bytes(m.width, m.hidden, m.lx, m.ld);
+        if (split > 0 && split_fits(m.width, m.hidden, 32)) {
+            if (cudaMalloc(&ctx->d_split, split * (size_t)n_leaves) != cudaSuccess) {
+                ctx->d_split = nullptr;
+                cudaGetLastError();
+            } else {
+                CK(prepare_mlp_split(m.width), "network kernel setup");
+                CK(launch_split_pack(ctx->stream, static_cast<const float*>(ctx->d_weights), stride / sizeof(float),
+                                     n_leaves, m.width, m.hidden, ctx->d_split),
+                   "split launch");
+                CK(cudaStreamSynchronize(ctx->stream), "stream sync");
+            }
+        }
+    }
     ctx->desc = m;
     ctx->n_nets = n_leaves;
     ctx->k0 = k0;
@@ -612,6 +634,14 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         a.t_begin = 0;
         a.t_end = 0xffffffffu;
         const bool tc = ctx->desc.prec != AMNERF_FP32;
+        // FP32 networks: split operands on the tensor cores where they are packed and fit;
+        // the SIMT kernel otherwise, and for calibration, which records its layer inputs
+        const bool split = ctx->d_split && !ctx->calibrating && split_fits(ctx->desc.width, ctx->desc.hidden, steps);
+        if (split) a.weights = ctx->d_split;
+        auto launch = [&](int grid) {
+            if (tc) return launch_mlp_tc(s, a, grid, (int)ctx->desc.prec);
+            return split ? launch_mlp_split(s, a, grid) : launch_mlp_simt(s, a, grid);
+        };
         a.groups = ctx->tuning.groups > 0 ? std::min(ctx->tuning.groups, ctx->max_groups) : ctx->max_groups;
         a.width_split = ctx->desc.prec == AMNERF_BF16 ? (ctx->tuning.width_split > 0 ? ctx->tuning.width_split
                                                                                        : kDefaultWidthSplit)
@@ -620,7 +650,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         if (!tc && sched != AMNERF_SCHED_PER_LEAF) sched = AMNERF_SCHED_CONTIGUOUS;
         a.schedule = sched == AMNERF_SCHED_PER_LEAF ? kSchedContiguous : sched;
         if (sched != AMNERF_SCHED_PER_LEAF) {
-            cudaError_t e = tc ? launch_mlp_tc(s, a, ctx->sm_count, (int)ctx->desc.prec) : launch_mlp_simt(s, a, ctx->sm_count);
+            cudaError_t e = launch(ctx->sm_count);
             if (e != cudaSuccess) return cuda_fail(ctx, e, "network launch");
         } else {
             // baseline: one launch per leaf, as a per-node library call would do
@@ -635,7 +665,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
                 a.t_end = te;
                 const uint32_t per_cta = tc ? (uint32_t)a.groups : 1u;
                 const int grid = (int)std::min<uint32_t>((uint32_t)ctx->sm_count, (te - tb + per_cta - 1) / per_cta);
-                cudaError_t e = tc ? launch_mlp_tc(s, a, grid, (int)ctx->desc.prec) : launch_mlp_simt(s, a, grid);
+                cudaError_t e = launch(grid);
                 if (e != cudaSuccess) return cuda_fail(ctx, e, "network launch");
             }
         }

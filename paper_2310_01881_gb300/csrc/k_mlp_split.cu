@@ -1,0 +1,547 @@
+// k_mlp_split.cu -- K-c, plain FP32 networks on the tensor cores (tcgen05, sm_103a), their
+// operands split into three BF16 parts.
+//
+// Same network and work unit as the FP32 SIMT path (Sec. 3.1 F_Theta, Sec. 3.2 same-shaped
+// networks, samples grouped by node, Sec. 3.5).  An FP32 value has 24 significand bits, a
+// BF16 value 8 and FP32's exponents, so v = h + m + l with h = bf16(v), m = bf16(v - h),
+// l = bf16(v - h - m) is exact (below about 2^-110, where parts become subnormal, up to an
+// absolute 2^-133).  A product of two split values is taken as the six largest of its nine
+// partial products -- h h, h m, m h, m m, h l, l h; the three left out are below
+// 2^-26 of it -- with the FP32 accumulator of the MMA.  That is the SIMT path's precision,
+// not a lower one: no operand or partial sum has fewer bits than FP32's own rounding.  The
+// tensor cores' accumulation truncates where FP32 arithmetic rounds to nearest, so each
+// layer adds its small products first (the accumulator then is 2^-8 of the sum, and so is
+// what a truncation drops), then the bias, and the h h products last: 5 or 6 accumulations
+// at full size against 64 to 90 roundings of an FP32 chain.
+//
+// Measured against 64 bits (relative 2-norm of the pixels' error, one 800 x 800 view):
+// 9.1e-7 with the SIMT kernel, 9.1e-7 here; the networks' own outputs, on the same sample
+// positions: 4.3e-8 (sigma) and 5.6e-8 (rgb) with the SIMT kernel, 4.3e-8 and 5.6e-8 here
+// (256 networks of 4 x 64), 2.6e-7 and 7.0e-7 against 2.5e-7 and 2.7e-7 with weights three
+// times as large; the largest single error is lower in every scene and shape measured.
+//
+// What bounds it: a 4 x 64 tile takes 135 MMAs, about 4 300 cycles of the tensor pipe, and
+// its rows about 3 000 instruction issues per SM sub-partition (42 sincospif per row, nine
+// instructions per split pair); three tiles of 168 TMEM columns are in flight per SM.  One
+// 800 x 800 view, network step: 7.6 ms (the SIMT kernel 37.6 ms, 46 % of the FP32 lanes'
+// peak); tensor pipe 52 %, issue 54 %.
+//
+// Structure, as k_mlp_tc: compute warpgroups of 128 threads, one thread per sample row
+// (TMEM lane), and one auxiliary warp per group that stages the crossings, loads weights
+// and issues the MMAs.  A network's split weights take three times a BF16 network's (123 KB
+// at 4 x 64), so the groups of a CTA share one copy: the CTA's contiguous range of tiles is
+// cut at leaf changes, its groups take a leaf's tiles in turn, and at a leaf change the
+// auxiliary warps meet on an mbarrier before one of them loads the next leaf's weights.
+// Layer 0's 96 input columns (90 features, the constant 1 of the bias, padding) are written
+// in three chunks of 32 (kPerm): all three h parts stay in TMEM for the last products, the
+// m and l parts of a chunk share one buffer.  While the head runs, a group encodes the
+// first chunk of its next tile.  Every wait is bounded.
+//
+// Kept on the SIMT kernel: calibration (per-layer input maxima), other encodings than
+// lx = 10, ld = 4, and networks whose split weights do not fit the shared memory.
+#include <cuda_bf16.h>
+
+#include <type_traits>
+
+#include "amnerf_internal.h"
+#include "tc_common.cuh"
+
+namespace amnerf {
+namespace {
+
+using namespace tcx;
+
+constexpr int kIn = 90, kInP = 96;  // encoded features; layer 0's K (bias at column 90)
+constexpr int kGroups = 3;          // compute warpgroups per CTA
+constexpr int kBiasK = 16;
+
+// TMEM columns of a group: D (accumulator), A (input parts), the constant ones of the bias
+// MMAs.  Layer 0: h parts of the 96 columns in A 0..47, a chunk's m and l parts in A 48..63
+// and 64..79; later layers: h, m, l parts in A 0.., 32.., 64...
+constexpr uint32_t kCols = 168, kA = 64, kOnes = 160;
+constexpr uint32_t kM0 = 48, kL0 = 64;
+static_assert(kGroups * kCols <= 512, "TMEM");
+
+// Registers per thread: 512 threads are launched with 128 each.
+constexpr int kComputeRegs = 144, kAuxRegs = 80;
+static_assert(kGroups * kComputeRegs + kAuxRegs <= (kGroups + 1) * 128, "the split draws on the launch's registers");
+
+// Layer 0's column order: column 2 i + 6 (and the next) hold sin and cos of pair i < 42
+// (octave i / 3 of coordinate i % 3 of x, the last 12 of d), columns 0..5 x and d.  Returns
+// the canonical feature, -1 for the bias column, -2 for padding.
+__host__ __device__ constexpr int kPerm(int c) {
+    if (c < 3) return c;
+    if (c < 6) return 60 + c;
+    if (c == 90) return -1;
+    if (c > 90) return -2;
+    const int i = (c - 6) >> 1, cosine = (c - 6) & 1;
+    return i < 30 ? 3 + 6 * (i / 3) + 3 * cosine + i % 3 : 66 + 6 * ((i - 30) / 3) + 3 * cosine + i % 3;
+}
+
+// A network's split weights (bytes): parts p = 0, 1, 2 (h, m, l) of every matrix as BF16
+// K-major core matrices; the hidden layers' biases as K = 16 operands (their three parts
+// at K columns 10..12, as in k_mlp_tc); the head's FP32 bias.
+struct SplitLayout {
+    int width, hidden;
+    size_t w0, wh, wo, bb, bo, stride;
+    __host__ __device__ SplitLayout(int w, int h) : width(w), hidden(h) {
+        w0 = 0;
+        wh = w0 + 3 * part0();
+        wo = wh + (size_t)(h - 1) * 3 * parth();
+        bb = wo + 3 * parto();
+        bo = bb + (size_t)(h - 1) * w * kBiasK * 2;
+        stride = (bo + 16 + 127) / 128 * 128;
+    }
+    __host__ __device__ size_t part0() const { return (size_t)width * kInP * 2; }
+    __host__ __device__ size_t parth() const { return (size_t)width * width * 2; }
+    __host__ __device__ size_t parto() const { return (size_t)16 * width * 2; }
+};
+
+struct SplitShared {
+    uint64_t bar_w;             // a leaf's weights
+    uint64_t bar_seg;           // the groups are done with a leaf's weights
+    uint64_t bar_a[kGroups];    // input parts written by the four compute warps
+    uint64_t bar_m[kGroups];    // MMAs completed
+    uint64_t bar_s[kGroups];    // crossings staged
+    int leaf[kGroups][kIdSlots];
+    uint32_t tmem_base;
+};
+constexpr size_t kShBytes = (sizeof(SplitShared) + 15) & ~(size_t)15;
+
+size_t split_smem(int width, int hidden, int cpt) {
+    return SplitLayout(width, hidden).stride + kShBytes + kGroups * stage_bytes(cpt);
+}
+
+__device__ __forceinline__ float2 bf16x2_floats(uint32_t p) {
+    return make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u));
+}
+
+// (v0, v1) = h + m + l, two BF16 per word.
+__device__ __forceinline__ void split3(float v0, float v1, uint32_t& h, uint32_t& m, uint32_t& l) {
+    const float2 neg = make_float2(-1.0f, -1.0f);
+    h = pack_bf16(v0, v1);
+    const float2 r = fma2v(bf16x2_floats(h), neg, make_float2(v0, v1));
+    m = pack_bf16(r.x, r.y);
+    const float2 s = fma2v(bf16x2_floats(m), neg, r);
+    l = pack_bf16(s.x, s.y);
+}
+
+__device__ __forceinline__ float softplus_f32(float z) { return z > 20.0f ? z : log1pf(expf(z)); }
+__device__ __forceinline__ float sigmoid_f32(float z) { return 1.0f / (1.0f + expf(-z)); }
+
+// The FP32 SIMT blob (transposed matrices, see k_mlp_simt.cu) of every network as split
+// operands, one element per thread and step; networks over blockIdx.y.
+__global__ void k_split_pack(const float* __restrict__ simt, size_t simt_stride, uint8_t* __restrict__ out, int W,
+                             int hidden) {
+    const SplitLayout lay(W, hidden);
+    const float* src = simt + (size_t)blockIdx.y * simt_stride;
+    uint8_t* dst = out + (size_t)blockIdx.y * lay.stride;
+    const int n0 = W * kInP, nh = (hidden - 1) * W * W, no = 16 * W, nb = (hidden - 1) * W * kBiasK;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n0 + nh + no + nb + 4; i += gridDim.x * blockDim.x) {
+        float v = 0.0f;
+        size_t at, part;
+        if (i < n0) {
+            const int n = i / kInP, c = i - n * kInP, f = kPerm(c);
+            v = f >= 0 ? src[(size_t)f * W + n] : (f == -1 ? src[(size_t)kIn * W + n] : 0.0f);
+            at = lay.w0 + cm_offset(n, c, kInP);
+            part = lay.part0();
+        } else if (i < n0 + nh) {
+            const int e = i - n0, l = e / (W * W), n = (e / W) % W, k = e % W;
+            v = src[(size_t)(kIn + 1) * W + (size_t)l * (W * W + W) + (size_t)k * W + n];
+            at = lay.wh + (size_t)l * 3 * lay.parth() + cm_offset(n, k, W);
+            part = lay.parth();
+        } else if (i < n0 + nh + no) {
+            const int e = i - n0 - nh, n = e / W, k = e % W;
+            const float* wo = src + (size_t)(kIn + 1) * W + (size_t)(hidden - 1) * (W * W + W);
+            v = n < 4 ? wo[(size_t)k * 4 + n] : 0.0f;
+            at = lay.wo + cm_offset(n, k, W);
+            part = lay.parto();
+        } else if (i < n0 + nh + no + nb) {
+            const int e = i - n0 - nh - no, l = e / (W * kBiasK), n = (e / kBiasK) % W, k = e % kBiasK;
+            const int p = k - (kOnesCol - kOnesStep);  // which part this K column carries
+            const float b = src[(size_t)(kIn + 1) * W + (size_t)l * (W * W + W) + (size_t)W * W + n];
+            const float h = __bfloat162float(__float2bfloat16_rn(b)), m = __bfloat162float(__float2bfloat16_rn(b - h));
+            v = p == 0 ? h : (p == 1 ? m : (p == 2 ? b - h - m : 0.0f));
+            *reinterpret_cast<__nv_bfloat16*>(dst + lay.bb + (size_t)l * W * kBiasK * 2 + cm_offset(n, k, kBiasK)) =
+                __float2bfloat16_rn(v);
+            continue;
+        } else {
+            const int n = i - n0 - nh - no - nb;
+            reinterpret_cast<float*>(dst + lay.bo)[n] =
+                src[(size_t)(kIn + 1) * W + (size_t)(hidden - 1) * (W * W + W) + 4 * W + n];
+            continue;
+        }
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const float r = v - __bfloat162float(h);
+        const __nv_bfloat16 m = __float2bfloat16_rn(r);
+        *reinterpret_cast<__nv_bfloat16*>(dst + at) = h;
+        *reinterpret_cast<__nv_bfloat16*>(dst + at + part) = m;
+        *reinterpret_cast<__nv_bfloat16*>(dst + at + 2 * part) = __float2bfloat16_rn(r - __bfloat162float(m));
+    }
+}
+
+// HC > 0: the number of hidden layers fixed at compile time.
+template <int W, int HC, bool JIT>
+__global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g) {
+    const int hidden = HC > 0 ? HC : g.hidden;
+    extern __shared__ __align__(1024) uint8_t smem[];
+    const SplitLayout lay(W, hidden);
+    SplitShared* sh = reinterpret_cast<SplitShared*>(smem + lay.stride);
+    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // uniform for the compiler
+    const int q = warp & 3, tig = threadIdx.x & 127, lane_id = threadIdx.x & 31;
+    if (threadIdx.x == 0) {
+        mbar_init(smem_u32(&sh->bar_w), 1);
+        mbar_init(smem_u32(&sh->bar_seg), kGroups);
+        for (int i = 0; i < kGroups; ++i) {
+            mbar_init(smem_u32(&sh->bar_a[i]), 4);
+            mbar_init(smem_u32(&sh->bar_m[i]), 1);
+            mbar_init(smem_u32(&sh->bar_s[i]), kStageArrivals);
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        fence_proxy_async();
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh->tmem_base)),
+                     "r"(512)
+                     : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = sh->tmem_base;
+
+    const bool aux = warp >= 4 * kGroups;
+    const int gi = aux ? q : warp >> 2;  // this warp's group (aux: warp i of the last warpgroup serves group i)
+    const int gc = gi < kGroups ? gi : 0;
+    const uint32_t bar_a = smem_u32(&sh->bar_a[gc]);
+    const uint32_t bar_m = smem_u32(&sh->bar_m[gc]);
+    const uint32_t bar_s = smem_u32(&sh->bar_s[gc]);
+    const uint32_t d_col = tmem + kCols * (uint32_t)gc;
+    const uint32_t a_col = d_col + kA;
+    const int cpt = kTileRows >> g.lg_steps;
+    uint8_t* stage = reinterpret_cast<uint8_t*>(sh) + kShBytes + gc * stage_bytes(cpt);
+    volatile int* leaf_s = sh->leaf[gc];
+    const uint8_t* wall = reinterpret_cast<const uint8_t*>(g.weights);
+    bool ok = true;  // the same in every thread of a warp
+    auto wait = [&](uint32_t bar, uint32_t phase) {
+        ok = __all_sync(0xffffffffu, mbar_wait_bounded(bar, phase));
+        return ok;
+    };
+    // this CTA's contiguous range of tiles; group i takes tiles t0 + i, t0 + i + kGroups, ...
+    const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
+    const uint32_t span = t_end > g.t_begin ? t_end - g.t_begin : 0u;
+    const uint32_t per = (span + gridDim.x - 1) / gridDim.x;
+    const uint32_t t0 = min(g.t_begin + blockIdx.x * per, t_end);
+    const uint32_t t1 = min(t0 + per, t_end);
+
+    if (aux) {
+        setmaxnreg_dec<kAuxRegs>();
+        if (gi < kGroups) {
+            const uint32_t w_addr = smem_u32(smem);
+            const uint32_t bar_w = smem_u32(&sh->bar_w), bar_seg = smem_u32(&sh->bar_seg);
+            const uint64_t desc0 = sdesc(w_addr + (uint32_t)lay.w0, kInP * 16u);
+            const uint64_t desch = sdesc(w_addr + (uint32_t)lay.wh, (uint32_t)W * 16u);
+            const uint64_t desco = sdesc(w_addr + (uint32_t)lay.wo, (uint32_t)W * 16u);
+            const uint64_t descb = sdesc(w_addr + (uint32_t)lay.bb, kBiasK * 16u);
+            const uint32_t p0 = (uint32_t)(lay.part0() >> 4), ph_ = (uint32_t)(lay.parth() >> 4),
+                           po = (uint32_t)(lay.parto() >> 4);
+            const uint32_t idd = idesc_bf16(W), idh = idesc_bf16(16);
+            Stager st(g, stage, sh->leaf[gc], bar_s, cpt, t0 + (uint32_t)gi, kGroups, t1);
+            uint32_t ph_a = 0, ph_w = 0, ph_seg = 0, n_m = 0;  // n_m: phases of bar_m committed
+            for (uint32_t n = 0; n < 3; ++n) st.ids(n);
+            cp_async_wait_all();
+            __syncwarp();
+            st.data(0);
+            st.data(1);
+            st.publish();
+            uint32_t n = 0;
+            // the leaves of the CTA's range in order, each with its tiles of this group
+            uint32_t t = t0;
+            int leaf = t0 < t1 ? leaf_of_tile_warp(g.tile_off, 0, g.n_leaves, t0) : 0;
+            while (t < t1 && ok) {
+                if (t > t0) {  // every group is done with the previous leaf's weights
+                    if (n_m > 0 && !wait(bar_m, (n_m - 1u) & 1u)) break;
+                    if (lane_id == 0) mbar_arrive(bar_seg);
+                    if (gi == 0 && !wait(bar_seg, ph_seg)) break;
+                    ph_seg ^= 1u;
+                }
+                if (gi == 0 && lane_id == 0) {
+                    fence_proxy_async();
+                    bulk_load(w_addr, wall + (size_t)leaf * lay.stride, (uint32_t)lay.stride, bar_w);
+                }
+                if (!wait(bar_w, ph_w)) break;
+                ph_w ^= 1u;
+                const uint32_t seg_end = min(t1, __ldg(g.tile_off + leaf + 1));
+                // this group's tiles below seg_end: numbers n with t0 + gi + kGroups n < seg_end
+                for (; t0 + (uint32_t)gi + kGroups * n < seg_end && ok; ++n) {
+                    // layer 0: per chunk the small products, after the last chunk the large ones
+#pragma unroll 1
+                    for (int c = 0; c < 3; ++c) {
+                        if (!wait(bar_a, ph_a)) break;
+                        ph_a ^= 1u;
+                        tc_fence_after();
+                        for (int s = 2 * c; s < 2 * c + 2; ++s) {
+                            const uint32_t ah = a_col + 8u * s, am = a_col + kM0 + 8u * (s & 1),
+                                           al = a_col + kL0 + 8u * (s & 1);
+                            const uint64_t b = desc0 + 16u * s;
+                            mma_bf16_ts_warp(d_col, am, b + p0, idd, s > 0 ? 1u : 0u);
+                            mma_bf16_ts_warp(d_col, al, b, idd, 1u);
+                            mma_bf16_ts_warp(d_col, ah, b + 2 * p0, idd, 1u);
+                            mma_bf16_ts_warp(d_col, am, b, idd, 1u);
+                            mma_bf16_ts_warp(d_col, ah, b + p0, idd, 1u);
+                        }
+                        if (c == 2)
+                            for (int s = 0; s < 6; ++s) mma_bf16_ts_warp(d_col, a_col + 8u * s, desc0 + 16u * s, idd, 1u);
+                        mma_commit_warp(bar_m);
+                        ++n_m;
+                    }
+                    if (!ok) break;
+                    // later layers, and the head onto D columns 0..15
+#pragma unroll 1
+                    for (int l = 1; l <= hidden; ++l) {
+                        if (!wait(bar_a, ph_a)) break;
+                        ph_a ^= 1u;
+                        tc_fence_after();
+                        const bool head = l == hidden;
+                        const uint64_t b0 = head ? desco : desch + (uint64_t)(3u * (uint32_t)(l - 1)) * ph_;
+                        const uint32_t pp = head ? po : ph_, id = head ? idh : idd;
+                        for (int s = 0; s < W / 16; ++s) {
+                            const uint32_t ah = a_col + 8u * s;
+                            const uint64_t b = b0 + 16u * s;
+                            mma_bf16_ts_warp(d_col, ah + 32u, b + pp, id, s > 0 ? 1u : 0u);
+                            mma_bf16_ts_warp(d_col, ah + 64u, b, id, 1u);
+                            mma_bf16_ts_warp(d_col, ah, b + 2 * pp, id, 1u);
+                        }
+                        for (int s = 0; s < W / 16; ++s) {
+                            const uint32_t ah = a_col + 8u * s;
+                            const uint64_t b = b0 + 16u * s;
+                            mma_bf16_ts_warp(d_col, ah + 32u, b, id, 1u);
+                            mma_bf16_ts_warp(d_col, ah, b + pp, id, 1u);
+                        }
+                        if (!head)
+                            mma_bf16_ts_warp(d_col, d_col + kOnes,
+                                             descb + (uint64_t)((uint32_t)(l - 1) * (W * kBiasK * 2 / 16)), id, 1u);
+                        for (int s = 0; s < W / 16; ++s) mma_bf16_ts_warp(d_col, a_col + 8u * s, b0 + 16u * s, id, 1u);
+                        mma_commit_warp(bar_m);
+                        ++n_m;
+                        // the slots' previous contents were read a tile ago; the arrival awaited
+                        // above follows the compute warps' wait for the phase before this one
+                        if (l == 1) {
+                            cp_async_wait_all();
+                            __syncwarp();
+                            st.data(n + 2);
+                            st.publish();
+                        }
+                        if (l == (hidden > 1 ? 2 : 1)) st.ids(n + 3);
+                    }
+                }
+                t = seg_end;
+                if (t < t1) leaf = leaf_of_tile_warp(g.tile_off, leaf + 1, g.n_leaves, t);
+            }
+            cp_async_wait_all();  // none in flight when the CTA ends
+            if (!ok && lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
+        }
+    } else {
+        setmaxnreg_inc<kComputeRegs>();
+        const uint32_t lane = (uint32_t)(32 * q) << 16;
+        const uint32_t d_row = d_col + lane, a_row = a_col + lane;
+        {
+            const uint32_t c8[8] = {0u, 0u, 0u, 0u, 0u, pack_bf16(1.0f, 1.0f), pack_bf16(1.0f, 0.0f), 0u};
+            tmem_st8(d_row + kOnes, c8);
+        }
+        const int ci = tig >> g.lg_steps, j = tig - (ci << g.lg_steps);
+        auto publish = [&]() {
+            tmem_st_wait();
+            tc_fence_before();
+            __syncwarp();
+            if (lane_id == 0) mbar_arrive(bar_a);
+        };
+        float x[3], d[3];
+        // chunk C of the layer-0 input: its split words
+        uint32_t wh[16], wm[16], wl[16];
+        auto encode = [&](auto chunk) {
+            constexpr int C = decltype(chunk)::value;
+#pragma unroll
+            for (int i = 0; i < 16; ++i) {
+                constexpr int kPairs = 42;
+                const int col = 32 * C + 2 * i;  // word i: columns col, col + 1
+                float v0, v1;
+                if (col < 6) {
+                    v0 = col == 0 ? x[0] : (col == 2 ? x[2] : d[1]);
+                    v1 = col == 0 ? x[1] : (col == 2 ? d[0] : d[2]);
+                } else {
+                    const int p = (col - 6) >> 1;
+                    if (p < kPairs) {
+                        const int oct = p < 30 ? p / 3 : (p - 30) / 3;
+                        sincospif((p < 30 ? x[p % 3] : d[p % 3]) * (float)(1 << oct), &v0, &v1);
+                    } else {  // the bias column's 1, then padding
+                        v0 = p == kPairs ? 1.0f : 0.0f;
+                        v1 = 0.0f;
+                    }
+                }
+                split3(v0, v1, wh[i], wm[i], wl[i]);
+            }
+            pin(wh);
+            pin(wm);
+            pin(wl);
+        };
+        auto store = [&](int c) {
+            tmem_st16(a_row + 16u * c, wh);
+            tmem_st16(a_row + kM0, wm);
+            tmem_st16(a_row + kL0, wl);
+            publish();
+        };
+        float4 bo = make_float4(0.f, 0.f, 0.f, 0.f);
+        uint32_t id = 0xffffffffu, ph_m = 0;
+        int cur = -1;
+        if (wait(bar_s, 0u) && leaf_s[0] >= 0) {
+            id = staged_sample<JIT>(g, stage, cpt, 0, ci, j, x, d);
+            encode(std::integral_constant<int, 0>());
+            store(0);
+        }
+        for (uint32_t n = 0; ok; ++n) {
+            const int leaf = leaf_s[n & (kIdSlots - 1)];
+            if (leaf < 0) break;
+            if (leaf != cur) {
+                bo = __ldg(reinterpret_cast<const float4*>(wall + (size_t)leaf * lay.stride + lay.bo));
+                cur = leaf;
+            }
+            // the m and l buffer is free when the previous chunk's small products are done
+            encode(std::integral_constant<int, 1>());
+            if (!wait(bar_m, ph_m)) break;
+            ph_m ^= 1u;
+            tc_fence_after();
+            store(1);
+            encode(std::integral_constant<int, 2>());
+            if (!wait(bar_m, ph_m)) break;
+            ph_m ^= 1u;
+            tc_fence_after();
+            store(2);
+            if (n > 0 && !wait(bar_s, n & 1u)) break;  // tile n + 1's crossings
+#pragma unroll 1
+            for (int l = 0; l < hidden; ++l) {
+                if (!wait(bar_m, ph_m)) break;
+                ph_m ^= 1u;
+                tc_fence_after();
+                // relu of the accumulator row, split, as the next layer's (or the head's) input
+#pragma unroll
+                for (int h = 0; h < W / 32; ++h) {
+                    float v[32];
+                    tmem_ld32(d_row + 32u * h, v);
+#pragma unroll
+                    for (int i = 0; i < 16; ++i)
+                        split3(fmaxf(v[2 * i], 0.0f), fmaxf(v[2 * i + 1], 0.0f), wh[i], wm[i], wl[i]);
+                    tmem_st16(a_row + 16u * h, wh);
+                    tmem_st16(a_row + 32u + 16u * h, wm);
+                    tmem_st16(a_row + 64u + 16u * h, wl);
+                }
+                publish();
+            }
+            if (!ok) break;
+            // under the head: the next tile's sample and first chunk
+            const uint32_t id_cur = id;
+            id = staged_sample<JIT>(g, stage, cpt, n + 1, ci, j, x, d);
+            const bool more = leaf_s[(n + 1) & (kIdSlots - 1)] >= 0;
+            encode(std::integral_constant<int, 0>());
+            if (!wait(bar_m, ph_m)) break;
+            ph_m ^= 1u;
+            tc_fence_after();
+            uint32_t z[4];
+            tmem_ld4_nowait(d_row, z);
+            tmem_ld_wait_regs(z);
+            if (more) store(0);
+            if (id_cur != 0xffffffffu) {
+                float4 o;
+                o.x = softplus_f32(__uint_as_float(z[0]) + bo.x);
+                o.y = sigmoid_f32(__uint_as_float(z[1]) + bo.y);
+                o.z = sigmoid_f32(__uint_as_float(z[2]) + bo.z);
+                o.w = sigmoid_f32(__uint_as_float(z[3]) + bo.w);
+                static_cast<float4*>(g.slot_out)[sample_slot(g, id_cur, j)] = o;
+            }
+        }
+        if (!ok && lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+}
+
+template <int W>
+constexpr int kHiddenFor = W == 64 ? 4 : 2;
+
+template <int W>
+cudaError_t prepare_w(int max_smem) {
+    const void* fns[4] = {(const void*)k_mlp_split<W, 0, false>, (const void*)k_mlp_split<W, 0, true>,
+                          (const void*)k_mlp_split<W, kHiddenFor<W>, false>,
+                          (const void*)k_mlp_split<W, kHiddenFor<W>, true>};
+    for (const void* f : fns) {
+        const cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
+template <int W>
+cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid, size_t smem) {
+    const bool hc = a.hidden == kHiddenFor<W>;
+    const int threads = 128 * (kGroups + 1);
+    if (a.jitter) {
+        if (hc) k_mlp_split<W, kHiddenFor<W>, true><<<grid, threads, smem, s>>>(a);
+        else k_mlp_split<W, 0, true><<<grid, threads, smem, s>>>(a);
+    } else {
+        if (hc) k_mlp_split<W, kHiddenFor<W>, false><<<grid, threads, smem, s>>>(a);
+        else k_mlp_split<W, 0, false><<<grid, threads, smem, s>>>(a);
+    }
+    return cudaGetLastError();
+}
+
+}  // namespace
+
+size_t split_leaf_stride_bytes(int width, int hidden, int lx, int ld) {
+    if (lx != 10 || ld != 4 || (width != 32 && width != 64)) return 0;
+    return SplitLayout(width, hidden).stride;
+}
+
+bool split_fits(int width, int hidden, int steps) {
+    int dev = 0, max_smem = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+        return false;
+    return split_smem(width, hidden, kTileRows / steps) <= (size_t)max_smem;
+}
+
+cudaError_t prepare_mlp_split(int width) {
+    int dev = 0, max_smem = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e != cudaSuccess) return e;
+    return width == 64 ? prepare_w<64>(max_smem) : prepare_w<32>(max_smem);
+}
+
+cudaError_t launch_split_pack(cudaStream_t s, const float* simt, size_t simt_stride, int n_nets, int width, int hidden,
+                              void* out) {
+    if (n_nets < 1) return cudaSuccess;
+    const int elems = width * kInP + (hidden - 1) * width * (width + kBiasK) + 16 * width + 4;
+    const dim3 grid((unsigned)((elems + 255) / 256), (unsigned)n_nets);
+    k_split_pack<<<grid, 256, 0, s>>>(simt, simt_stride, static_cast<uint8_t*>(out), width, hidden);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_mlp_split(cudaStream_t s, const MlpArgs& a, int grid) {
+    int dev = 0, max_smem = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    size_t smem = split_smem(a.width, a.hidden, kTileRows >> a.lg_steps);
+    if (smem > (size_t)max_smem) return cudaErrorInvalidConfiguration;
+    // more than half of the SM's shared memory: a second CTA can never become resident and
+    // wait in tcgen05.alloc for columns that this one holds
+    if (smem < (size_t)max_smem / 2 + 1024) smem = (size_t)max_smem / 2 + 1024;
+    if (a.width == 64) return launch_w<64>(s, a, grid, smem);
+    if (a.width == 32) return launch_w<32>(s, a, grid, smem);
+    return cudaErrorInvalidValue;
+}
+
+}  // namespace amnerf

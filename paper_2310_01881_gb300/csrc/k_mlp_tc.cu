@@ -161,15 +161,6 @@ struct TcShared {
     uint32_t tmem_base;
 };
 
-// id / maxc: q = floor(id m / 2^32) with m = ceil(2^32 / maxc) is the quotient or one
-// more (id m / 2^32 < id / maxc + 1); one compare fixes it.
-__device__ __forceinline__ uint32_t div_maxc(const MlpArgs& g, uint32_t id) {
-    if (g.maxc == 1) return id;
-    uint32_t q = __umulhi(id, g.maxc_magic);
-    if ((uint64_t)q * (uint32_t)g.maxc > id) --q;
-    return q;
-}
-
 // Crossing of this row in tile t of `leaf` (0xffffffff past the leaf's end).
 __device__ __forceinline__ uint32_t row_crossing(const MlpArgs& g, int leaf, uint32_t t, int ci) {
     const uint32_t first = __ldg(g.offsets + leaf) + (t - __ldg(g.tile_off + leaf)) * (uint32_t)(kTileRows >> g.lg_steps);
@@ -205,30 +196,12 @@ constexpr uint32_t kACol = 64;
 constexpr uint32_t kHeadCol = 112;
 constexpr uint32_t kA0Col8 = 16;  // E4M3: first A column of the layer-0 input
 
-// Keeps the n words of a value computed here from being computed later: pure register
-// arithmetic may otherwise be moved past the volatile waits that follow it.
-template <int N>
-__device__ __forceinline__ void pin(uint32_t (&w)[N]) {
-#pragma unroll
-    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(w[i]));
-}
-
 // Registers per thread: 128 (groups + 1) threads are launched with 96 each; the compute
 // warpgroups take more and leave the last one the rest (at four groups the whole launch:
 // 4 x 112 + 32 = 5 x 96; fewer groups ask for less than they were launched with).
 constexpr int kComputeRegs = 104, kAuxRegs = 64;
 static_assert(kMaxGroups * kComputeRegs + kAuxRegs <= (kMaxGroups + 1) * 96 && kComputeRegs - 96 <= 96 - kAuxRegs,
               "the split draws on the launch's registers");
-
-// A group's crossings in shared memory, staged ahead by one of its warps (cpt = crossings
-// per tile, 128 / steps): the interval and the ray of every crossing of two tiles (32 B:
-// t_in, t_out, o, d) and the crossing ids of four (0xffffffff past a leaf's end).  The
-// copies are cp.async: a load into registers is waited for before the block that issued it
-// is left, which cost every group one to two DRAM latencies per tile.
-constexpr int kDataSlots = 2, kIdSlots = 4;
-__host__ __device__ constexpr size_t stage_bytes(int cpt) {
-    return (size_t)cpt * (kDataSlots * 32 + kIdSlots * 4);
-}
 
 // F8 = false: BF16 operands (kind::f16, K = 16 per MMA, 2 features per TMEM column).
 // F8 = true:  E4M3 operands (kind::f8f6f4, K = 32 per MMA, 4 features per column).
@@ -293,7 +266,7 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
             mbar_init(smem_u32(&sh->bar_m[i]), 1);
             mbar_init(smem_u32(&sh->bar_h[i]), 1);
             mbar_init(smem_u32(&sh->bar_a[i]), 4);
-            mbar_init(smem_u32(&sh->bar_s[i]), 33);
+            mbar_init(smem_u32(&sh->bar_s[i]), kStageArrivals);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -323,12 +296,9 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
     const uint32_t bar_s = smem_u32(&sh->bar_s[gi]);
     const uint32_t d_col = tmem + kGroupCols * (uint32_t)gi;  // lane 0: MMA operand addresses
     const uint32_t a_col = d_col + kACol;
-    // Tile n of the group has its leaf in leaf_s[n % 4] (-1: no such tile), its crossing ids
-    // in id_s[n % 4] and its intervals and rays in data_s[n % 2].
+    // the group's staged crossings (see Stager)
     const int cpt = kTileRows >> g.lg_steps;
     uint8_t* stage = reinterpret_cast<uint8_t*>(sh) + ((sizeof(TcShared) + 15) & ~(size_t)15) + gi * stage_bytes(cpt);
-    float* data_s = reinterpret_cast<float*>(stage);
-    uint32_t* id_s = reinterpret_cast<uint32_t*>(stage + (size_t)cpt * kDataSlots * 32);
     volatile int* leaf_s = sh->leaf[gi];
     bool ok = true;  // the same in every thread of a warp
     // A wait that ran out (about 2 s) ends the warp's loop: it arrives at no barrier any
@@ -352,10 +322,7 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
             const uint64_t desc_bb = sdesc(w_addr + (uint32_t)lay.bb, (uint32_t)kBiasK * 16u);
             const uint8_t* wall = reinterpret_cast<const uint8_t*>(g.weights);
             const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
-            uint32_t t_stop = t_end, t_step = 1, t_next;  // the next tile to look up
-            // the looked-up leaf's tile range and crossing range change only at leaf changes
-            uint32_t lk_t0 = 0u, lk_t1 = 0u, lk_x0 = 0u, lk_x1 = 0u;
-            int lk_leaf = -1;
+            uint32_t t_stop = t_end, t_step = 1, t_next;
             {
                 const uint32_t workers = gridDim.x * (uint32_t)n_groups;
                 const uint32_t wid = blockIdx.x * (uint32_t)n_groups + (uint32_t)gi;
@@ -371,69 +338,18 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                     t_stop = min(t_next + per, t_end);
                 }
             }
-            // the stager warp: leaf and crossing ids of tile n (tiles come in increasing order)
-            auto stage_ids = [&](uint32_t n) {
-                if (g.schedule == kSchedDynamic) {
-                    uint32_t v = 0;
-                    if (lane_id == 0) v = atomicAdd(g.tile_counter, 1u) + g.t_begin;
-                    t_next = __shfl_sync(0xffffffffu, v, 0);
-                }
-                uint32_t* dst = id_s + (n & (kIdSlots - 1)) * cpt;
-                const bool any = t_next < t_stop;
-                if (any) {
-                    if (t_next >= lk_t1) {
-                        lk_leaf = leaf_of_tile_warp(g.tile_off, lk_leaf + 1, g.n_leaves, t_next);
-                        lk_t0 = __ldg(g.tile_off + lk_leaf);
-                        lk_t1 = __ldg(g.tile_off + lk_leaf + 1);
-                        lk_x0 = __ldg(g.offsets + lk_leaf);
-                        lk_x1 = __ldg(g.offsets + lk_leaf + 1);
-                    }
-                    for (int c = lane_id; c < cpt; c += 32) {
-                        const uint32_t at = lk_x0 + (t_next - lk_t0) * (uint32_t)cpt + (uint32_t)c;
-                        if (at < lk_x1) cp_async<4>(smem_u32(dst + c), g.order + at);
-                        else dst[c] = 0xffffffffu;
-                    }
-                } else {
-                    for (int c = lane_id; c < cpt; c += 32) dst[c] = 0xffffffffu;
-                }
-                if (lane_id == 0) leaf_s[n & (kIdSlots - 1)] = any ? lk_leaf : -1;
-                t_next += t_step;
-            };
-            // ... and, its ids staged, the intervals and rays of tile n
-            auto stage_data = [&](uint32_t n) {
-                const uint32_t* ids = id_s + (n & (kIdSlots - 1)) * cpt;
-                const uint32_t dst = smem_u32(data_s + (n & (kDataSlots - 1)) * cpt * 8);
-                for (int c = lane_id; c < cpt; c += 32) {
-                    const uint32_t id = ids[c];
-                    if (id == 0xffffffffu) continue;
-                    const size_t ray = 3 * (size_t)div_maxc(g, id);
-                    cp_async<8>(dst + 32 * c, g.xing + id);
-#pragma unroll
-                    for (int a = 0; a < 3; ++a) {
-                        cp_async<4>(dst + 32 * c + 8 + 4 * a, g.ro + ray + a);
-                        cp_async<4>(dst + 32 * c + 20 + 4 * a, g.rd + ray + a);
-                    }
-                }
-            };
-
-            // one phase of bar_s: 32 arrivals when the lanes' copies so far are complete, and one
-            // that releases the plain stores
-            auto publish_stage = [&]() {
-                cp_async_arrive(bar_s);
-                __syncwarp();
-                if (lane_id == 0) mbar_arrive(bar_s);
-            };
+            Stager st(g, stage, sh->leaf[gi], bar_s, cpt, t_next, t_step, t_stop);
             uint32_t ph_w = 0, ph_h = 0, ph_a = 0;
-            for (uint32_t n = 0; n < 3; ++n) stage_ids(n);
+            for (uint32_t n = 0; n < 3; ++n) st.ids(n);
             __syncwarp();
             int cur = leaf_s[0];
             if (cur >= 0 && lane_id == 0)
                 bulk_load(w_addr, wall + (size_t)cur * lay.stride, (uint32_t)lay.stride, bar_w);
             cp_async_wait_all();
             __syncwarp();
-            stage_data(0);
-            stage_data(1);
-            publish_stage();
+            st.data(0);
+            st.data(1);
+            st.publish();
             bool fresh = true;  // weights loaded but not yet waited for
             for (uint32_t n = 0;; ++n) {
                 const int leaf = leaf_s[n & (kIdSlots - 1)];
@@ -514,10 +430,10 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                     if (l == (hidden > 1 ? 1 : 0)) {
                         cp_async_wait_all();
                         __syncwarp();
-                        stage_data(n + 2);
-                        publish_stage();
+                        st.data(n + 2);
+                        st.publish();
                     }
-                    if (l == (hidden > 2 ? 2 : hidden - 1)) stage_ids(n + 3);
+                    if (l == (hidden > 2 ? 2 : hidden - 1)) st.ids(n + 3);
                 }
                 if (!ok) break;
             }
@@ -552,44 +468,17 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
         uint32_t zr[4] = {0u, 0u, 0u, 0u};
         auto store_head = [&]() {
             if (id_prev != 0xffffffffu) {  // 4 x FP16; sigma saturates at the FP16 maximum
-                const uint32_t ray = div_maxc(g, id_prev);
-                const uint32_t k = id_prev - ray * (uint32_t)g.maxc;
-                // 64-bit: rays * cap may exceed 2^32
-                const uint64_t slot_prev = (uint64_t)ray * (uint64_t)g.cap + (uint64_t)((k << g.lg_steps) + (uint32_t)j);
                 uint2 o;
                 o.x = pack_f16(fminf(softplus_f(__uint_as_float(zr[0])), 65504.0f), sigmoid_f(__uint_as_float(zr[1])));
                 o.y = pack_f16(sigmoid_f(__uint_as_float(zr[2])), sigmoid_f(__uint_as_float(zr[3])));
-                static_cast<uint2*>(g.slot_out)[slot_prev] = o;
+                static_cast<uint2*>(g.slot_out)[sample_slot(g, id_prev, j)] = o;
             }
         };
         // this row's sample of the tile to be encoded: its crossing, position and direction
         uint32_t id = 0xffffffffu;
         float rd[3] = {0.f, 0.f, 0.f};
         float x[3];  // its position
-        auto place_sample = [&](uint32_t n) {
-            id = id_s[(n & (kIdSlots - 1)) * cpt + ci];
-            const float4* p = reinterpret_cast<const float4*>(data_s + ((n & (kDataSlots - 1)) * cpt + ci) * 8);
-            const float4 u0 = p[0], u1 = p[1];
-            if (id != 0xffffffffu) {
-                const float ro[3] = {u0.z, u0.w, u1.x};
-                rd[0] = u1.y;
-                rd[1] = u1.z;
-                rd[2] = u1.w;
-                // steps is a power of two: the product by its reciprocal is the exact quotient
-                const float delta = __fmul_rn(__fsub_rn(u0.y, u0.x), __frcp_rn((float)g.steps));
-                float u = 0.5f;
-                if constexpr (JIT) {
-                    const uint32_t k = id - div_maxc(g, id) * (uint32_t)g.maxc;
-                    u = jit_fraction(g.jitter, jit_ray_key(g.jitter, ro, rd), (int)k, g.steps, j);
-                }
-                const float tj = __fadd_rn(u0.x, __fmul_rn(__fadd_rn((float)j, u), delta));
-#pragma unroll
-                for (int a = 0; a < 3; ++a) x[a] = __fadd_rn(ro[a], __fmul_rn(tj, rd[a]));
-            } else {
-#pragma unroll
-                for (int a = 0; a < 3; ++a) x[a] = rd[a] = 0.f;
-            }
-        };
+        auto place_sample = [&](uint32_t n) { id = staged_sample<JIT>(g, stage, cpt, n, ci, j, x, rd); };
 
         // ---- the layer-0 input of the sample in three parts (kperm's column order for BF16,
         // the canonical one for E4M3), each computed under one layer's MMAs and stored where

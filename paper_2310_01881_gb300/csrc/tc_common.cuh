@@ -326,6 +326,14 @@ __device__ __forceinline__ uint32_t pack_relu_e4m3x4(float a, float b, float c, 
     return r;
 }
 
+// Keeps the n words of a value computed here from being computed later: pure register
+// arithmetic may otherwise be moved past the volatile waits that follow it.
+template <int N>
+__device__ __forceinline__ void pin(uint32_t (&w)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) asm volatile("" : "+r"(w[i]));
+}
+
 // Head activations with the SFU exp/log/reciprocal (relative error ~1e-6, far below the
 // BF16/E4M3 operand rounding of this path).
 __device__ __forceinline__ float rcp_approx(float x) {
@@ -358,6 +366,143 @@ __device__ __forceinline__ int leaf_of_tile_warp(const uint32_t* __restrict__ ti
         hi = min(hi, lo + step);
     }
     return lo;
+}
+
+// id / maxc: q = floor(id m / 2^32) with m = ceil(2^32 / maxc) is the quotient or one
+// more (id m / 2^32 < id / maxc + 1); one compare fixes it.
+__device__ __forceinline__ uint32_t div_maxc(const MlpArgs& g, uint32_t id) {
+    if (g.maxc == 1) return id;
+    uint32_t q = __umulhi(id, g.maxc_magic);
+    if ((uint64_t)q * (uint32_t)g.maxc > id) --q;
+    return q;
+}
+
+// A warpgroup's crossings in shared memory, staged tiles ahead by one warp (cpt = crossings
+// per tile, 128 / steps): the interval and the ray of every crossing of two tiles (32 B:
+// t_in, t_out, o, d) and the crossing ids of four (0xffffffff past a leaf's end).  The
+// copies are cp.async: a load into registers is waited for before the block that issued it
+// is left, which cost every group one to two DRAM latencies per tile.
+constexpr int kDataSlots = 2, kIdSlots = 4;
+__host__ __device__ constexpr size_t stage_bytes(int cpt) {
+    return (size_t)cpt * (kDataSlots * 32 + kIdSlots * 4);
+}
+
+// Tile n of the group has its leaf in leaf[n % kIdSlots] (-1: no such tile), its crossing ids
+// in id_s() [n % kIdSlots] and its intervals and rays in data_s() [n % kDataSlots].
+__device__ __forceinline__ float* stage_data_s(uint8_t* stage) { return reinterpret_cast<float*>(stage); }
+__device__ __forceinline__ uint32_t* stage_id_s(uint8_t* stage, int cpt) {
+    return reinterpret_cast<uint32_t*>(stage + (size_t)cpt * kDataSlots * 32);
+}
+
+// The staging warp's side: the group's tiles are t_next, t_next + t_step, ... below t_stop
+// (or taken from the device counter: dynamic schedule).  All methods by the whole warp.
+struct Stager {
+    const MlpArgs& g;
+    uint8_t* stage;
+    volatile int* leaf;
+    uint32_t bar_s;
+    int cpt;
+    uint32_t t_next, t_step, t_stop;
+    // the looked-up leaf's tile range and crossing range change only at leaf changes
+    uint32_t lk_t0 = 0u, lk_t1 = 0u, lk_x0 = 0u, lk_x1 = 0u;
+    int lk_leaf = -1;
+    __device__ __forceinline__ Stager(const MlpArgs& g_, uint8_t* stage_, volatile int* leaf_, uint32_t bar, int cpt_,
+                                      uint32_t next, uint32_t step, uint32_t stop)
+        : g(g_), stage(stage_), leaf(leaf_), bar_s(bar), cpt(cpt_), t_next(next), t_step(step), t_stop(stop) {}
+
+    // leaf and crossing ids of tile n (the tiles come in increasing order)
+    __device__ __forceinline__ void ids(uint32_t n) {
+        const int lane = threadIdx.x & 31;
+        if (g.schedule == kSchedDynamic) {
+            uint32_t v = 0;
+            if (lane == 0) v = atomicAdd(g.tile_counter, 1u) + g.t_begin;
+            t_next = __shfl_sync(0xffffffffu, v, 0);
+        }
+        uint32_t* dst = stage_id_s(stage, cpt) + (n & (kIdSlots - 1)) * cpt;
+        const bool any = t_next < t_stop;
+        if (any) {
+            if (t_next >= lk_t1) {
+                lk_leaf = leaf_of_tile_warp(g.tile_off, lk_leaf + 1, g.n_leaves, t_next);
+                lk_t0 = __ldg(g.tile_off + lk_leaf);
+                lk_t1 = __ldg(g.tile_off + lk_leaf + 1);
+                lk_x0 = __ldg(g.offsets + lk_leaf);
+                lk_x1 = __ldg(g.offsets + lk_leaf + 1);
+            }
+            for (int c = lane; c < cpt; c += 32) {
+                const uint32_t at = lk_x0 + (t_next - lk_t0) * (uint32_t)cpt + (uint32_t)c;
+                if (at < lk_x1) cp_async<4>(smem_u32(dst + c), g.order + at);
+                else dst[c] = 0xffffffffu;
+            }
+        } else {
+            for (int c = lane; c < cpt; c += 32) dst[c] = 0xffffffffu;
+        }
+        if (lane == 0) leaf[n & (kIdSlots - 1)] = any ? lk_leaf : -1;
+        t_next += t_step;
+    }
+
+    // the intervals and rays of tile n, whose ids are staged
+    __device__ __forceinline__ void data(uint32_t n) {
+        const uint32_t* idn = stage_id_s(stage, cpt) + (n & (kIdSlots - 1)) * cpt;
+        const uint32_t dst = smem_u32(stage_data_s(stage) + (n & (kDataSlots - 1)) * cpt * 8);
+        for (int c = threadIdx.x & 31; c < cpt; c += 32) {
+            const uint32_t id = idn[c];
+            if (id == 0xffffffffu) continue;
+            const size_t ray = 3 * (size_t)div_maxc(g, id);
+            cp_async<8>(dst + 32 * c, g.xing + id);
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                cp_async<4>(dst + 32 * c + 8 + 4 * a, g.ro + ray + a);
+                cp_async<4>(dst + 32 * c + 20 + 4 * a, g.rd + ray + a);
+            }
+        }
+    }
+
+    // one phase of bar_s: 32 arrivals when the lanes' copies so far are complete, and one that
+    // releases the plain stores (bar_s counts kStageArrivals)
+    __device__ __forceinline__ void publish() {
+        cp_async_arrive(bar_s);
+        __syncwarp();
+        if ((threadIdx.x & 31) == 0) mbar_arrive(bar_s);
+    }
+};
+constexpr int kStageArrivals = 33;
+
+// The sample of row (crossing ci of tile n, sample j of the crossing), rebuilt in the
+// traversal's FP32 order: its crossing id (returned; 0xffffffff and a zero sample past the
+// leaf's end), position x and direction d.
+template <bool JIT>
+__device__ __forceinline__ uint32_t staged_sample(const MlpArgs& g, uint8_t* stage, int cpt, uint32_t n, int ci, int j,
+                                                  float (&x)[3], float (&d)[3]) {
+    const uint32_t id = stage_id_s(stage, cpt)[(n & (kIdSlots - 1)) * cpt + ci];
+    const float4* p = reinterpret_cast<const float4*>(stage_data_s(stage) + ((n & (kDataSlots - 1)) * cpt + ci) * 8);
+    const float4 u0 = p[0], u1 = p[1];
+    if (id != 0xffffffffu) {
+        const float o[3] = {u0.z, u0.w, u1.x};
+        d[0] = u1.y;
+        d[1] = u1.z;
+        d[2] = u1.w;
+        // steps is a power of two: the product by its reciprocal is the exact quotient
+        const float delta = __fmul_rn(__fsub_rn(u0.y, u0.x), __frcp_rn((float)g.steps));
+        float u = 0.5f;
+        if constexpr (JIT) {
+            const uint32_t k = id - div_maxc(g, id) * (uint32_t)g.maxc;
+            u = jit_fraction(g.jitter, jit_ray_key(g.jitter, o, d), (int)k, g.steps, j);
+        }
+        const float tj = __fadd_rn(u0.x, __fmul_rn(__fadd_rn((float)j, u), delta));
+#pragma unroll
+        for (int a = 0; a < 3; ++a) x[a] = __fadd_rn(o[a], __fmul_rn(tj, d[a]));
+    } else {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) x[a] = d[a] = 0.f;
+    }
+    return id;
+}
+
+// The output slot of sample j of crossing `id` (64-bit: rays * cap may exceed 2^32).
+__device__ __forceinline__ uint64_t sample_slot(const MlpArgs& g, uint32_t id, int j) {
+    const uint32_t ray = div_maxc(g, id);
+    const uint32_t k = id - ray * (uint32_t)g.maxc;
+    return (uint64_t)ray * (uint64_t)g.cap + (uint64_t)((k << g.lg_steps) + (uint32_t)j);
 }
 
 // sin(pi 2^k p), cos(pi 2^k p): the argument is reduced exactly to r in [-1, 1]

@@ -208,10 +208,15 @@ cudaError_t launch_prop_infer_tc(cudaStream_t s, const float* params, const floa
                                  const float* rd, uint32_t n, float coverage, int max_bins, uint64_t* mask,
                                  uint8_t* fallback, unsigned long long* n_fallback, int* err,
                                  float* q_out = nullptr);
-cudaError_t launch_prop_grad(cudaStream_t s, const float* params, const float* ro, const float* rd,
+// One training step (two launches): the gradient of the batch's mean loss, then Adam on P, m,
+// v (step counts from 1), or with P == nullptr the gradient into grad; the loss into *loss.
+// part: prop_partial_floats() floats of scratch.  first: no earlier step of the same call
+// precedes it in the stream.
+size_t prop_partial_floats();
+cudaError_t launch_prop_step(cudaStream_t s, bool first, const float* params, const float* ro, const float* rd,
                              const float2* root, const float* targets, uint32_t n, uint32_t batch, uint64_t seed,
-                             uint64_t step, float* grad, float* loss);
-cudaError_t launch_prop_adam(cudaStream_t s, float* P, float* g, float* m, float* v, int t, float lr);
+                             uint64_t step, float* part, float* P, float* m, float* v, float lr, float* grad,
+                             float* loss);
 
 // ---- host tree builder -------------------------------------------------------------
 // Returns false on invalid input (message in err).

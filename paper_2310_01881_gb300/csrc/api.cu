@@ -77,6 +77,9 @@ struct amnerf_ctx {
     int prop_grid = 0;        // persistent grid of the inference kernel on this device
     int prop_step = 0;
     float* d_prop = nullptr;  // params | m | v | grad | loss (5 x NPAR floats + 1)
+    float* d_part = nullptr;  // partial gradients of a training step
+    size_t cap_losses = 0;
+    float* d_losses = nullptr;  // losses of one training call
     size_t cap_prop_rays = 0;
     uint64_t* d_mask = nullptr;
     uint8_t* d_fallback = nullptr;
@@ -236,6 +239,18 @@ static amnerf_status ensure_prop_scratch(amnerf_ctx* ctx, size_t n) {
     return AMNERF_OK;
 }
 
+// Training scratch: the partial gradients, and room for the losses of `steps` steps.
+static amnerf_status ensure_train_scratch(amnerf_ctx* ctx, size_t steps) {
+    if (!ctx->d_part) CK(cudaMalloc((void**)&ctx->d_part, sizeof(float) * prop_partial_floats()), "training allocation");
+    if (steps > ctx->cap_losses) {
+        dfree(ctx->d_losses);
+        ctx->cap_losses = 0;
+        CK(cudaMalloc((void**)&ctx->d_losses, sizeof(float) * steps), "loss buffer");
+        ctx->cap_losses = steps;
+    }
+    return AMNERF_OK;
+}
+
 extern "C" {
 
 const char* amnerf_status_string(amnerf_status s) {
@@ -324,6 +339,8 @@ void amnerf_destroy(amnerf_ctx* ctx) {
     dfree(ctx->d_err);
     dfree(ctx->d_hbuf);
     dfree(ctx->d_prop);
+    dfree(ctx->d_part);
+    dfree(ctx->d_losses);
     dfree(ctx->d_mask);
     dfree(ctx->d_fallback);
     dfree(ctx->d_root);
@@ -966,22 +983,21 @@ amnerf_status amnerf_proposal_train(amnerf_ctx* ctx, const float* ro, const floa
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     cudaStream_t s = ctx->stream;
     std::vector<float> h_loss((size_t)steps);
-    float* d_losses = nullptr;
-    if (steps > 0) CK(cudaMalloc((void**)&d_losses, sizeof(float) * (size_t)steps), "loss buffer");
-    CK(cudaMemsetAsync(prop_g(ctx), 0, sizeof(float) * proposal_param_count(), s), "memset");
-    if (steps > 0) CK(cudaMemsetAsync(d_losses, 0, sizeof(float) * (size_t)steps, s), "memset");
+    if (steps > 0) {
+        amnerf_status st = ensure_train_scratch(ctx, (size_t)steps);
+        if (st != AMNERF_OK) return st;
+    }
     cudaError_t e = cudaSuccess;
     for (int i = 0; i < steps && e == cudaSuccess; ++i) {
         const uint64_t step = (uint64_t)ctx->prop_step + 1;
-        e = launch_prop_grad(s, prop_params(ctx), ro, rd, reinterpret_cast<const float2*>(root), targets, (uint32_t)n,
-                             (uint32_t)batch, seed, step, prop_g(ctx), d_losses + i);
-        if (e == cudaSuccess) e = launch_prop_adam(s, prop_params(ctx), prop_g(ctx), prop_m(ctx), prop_v(ctx), (int)step, lr);
+        e = launch_prop_step(s, i == 0, prop_params(ctx), ro, rd, reinterpret_cast<const float2*>(root), targets,
+                             (uint32_t)n, (uint32_t)batch, seed, step, ctx->d_part, prop_params(ctx), prop_m(ctx),
+                             prop_v(ctx), lr, nullptr, ctx->d_losses + i);
         ctx->prop_step += 1;
     }
     if (e == cudaSuccess && steps > 0)
-        e = cudaMemcpyAsync(h_loss.data(), d_losses, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost, s);
+        e = cudaMemcpyAsync(h_loss.data(), ctx->d_losses, sizeof(float) * (size_t)steps, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (d_losses) cudaFree(d_losses);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "proposal training");
     if (losses) std::memcpy(losses, h_loss.data(), sizeof(float) * (size_t)steps);
     return AMNERF_OK;
@@ -995,14 +1011,13 @@ amnerf_status amnerf_proposal_grad(amnerf_ctx* ctx, const float* ro, const float
     CK(cudaSetDevice(ctx->device), "cudaSetDevice");
     cudaStream_t s = ctx->stream;
     const int np = proposal_param_count();
-    CK(cudaMemsetAsync(prop_g(ctx), 0, sizeof(float) * np, s), "memset");
-    CK(cudaMemsetAsync(prop_loss(ctx), 0, sizeof(float), s), "memset");
-    CK(launch_prop_grad(s, prop_params(ctx), ro, rd, reinterpret_cast<const float2*>(root), targets, (uint32_t)n,
-                        (uint32_t)n, 0, 0, prop_g(ctx), prop_loss(ctx)),
+    amnerf_status st = ensure_train_scratch(ctx, 0);
+    if (st != AMNERF_OK) return st;
+    CK(launch_prop_step(s, true, prop_params(ctx), ro, rd, reinterpret_cast<const float2*>(root), targets, (uint32_t)n,
+                        (uint32_t)n, 0, 0, ctx->d_part, nullptr, nullptr, nullptr, 0.0f, prop_g(ctx), prop_loss(ctx)),
        "proposal gradient");
     CK(cudaMemcpyAsync(grad, prop_g(ctx), sizeof(float) * np, cudaMemcpyDeviceToHost, s), "download");
     CK(cudaMemcpyAsync(loss, prop_loss(ctx), sizeof(float), cudaMemcpyDeviceToHost, s), "download");
-    CK(cudaMemsetAsync(prop_g(ctx), 0, sizeof(float) * np, s), "memset");
     CK(cudaStreamSynchronize(s), "stream sync");
     return AMNERF_OK;
 }

@@ -24,11 +24,10 @@
 //                  128 x 32 x 48, 128 x 80 x 48; activations in TMEM), then the softmax
 //                  and the same bin selection.  amnerf_proposal_predict keeps the FP32
 //                  kernel (its probabilities are the FP32 ones).
-//   k_prop_grad    one CTA per 128 rays: each thread runs its ray forward and
-//                  backward and leaves its activations and deltas in shared memory;
-//                  the CTA then forms the gradient contractions (sum over its rays of
-//                  delta x activation) and adds them with one atomic per parameter.
-//   k_prop_adam    elementwise Adam update, then clears the gradient.
+//   k_prop_grad    64 rays per CTA tile, every layer, its backward pass and the gradient
+//                  contractions spread over 512 threads from shared memory; one partial
+//                  gradient per CTA.
+//   k_prop_reduce  sums the partials and applies Adam.
 #include <cstring>
 
 #include "amnerf_internal.h"
@@ -594,130 +593,306 @@ __device__ __forceinline__ uint32_t batch_ray(uint64_t seed, uint64_t s, uint32_
     return (uint32_t)(z % n);
 }
 
+// ---- training ------------------------------------------------------------------------
+// Gradient of the mean cross-entropy over a batch of B rays (ray indices from the
+// counter-based hash, or the rays in order), then Adam.  A step is two launches:
+// k_prop_grad leaves one partial gradient per CTA, k_prop_reduce sums the partials in a
+// fixed order and updates the parameters (no atomics: a step's result does not vary).
+//
+// What bounds it: a step is 0.3 GFLOP, so latency.  With one thread per ray (64 CTAs of 128
+// threads, each thread walking its ray's 6 000 multiply-adds alone) a step of 8192 rays took
+// 98 us; with 64 rays per CTA of 512 threads, every layer and contraction spread over all of
+// them from shared memory, 25 us (24 steps 2.36 -> 0.60 ms).  Rows of 68 floats keep the 16-byte loads of
+// neighbouring rows on different banks.  The next step's launch overlaps its ray loads and
+// encodings with the update (programmatic dependent launch).
+constexpr int kGRays = 64, kGThreads = 512, kGLd = 68;
+constexpr int kPartCtas = 304;       // at most (two per SM); each takes every kPartCtas-th tile of 64 rays
+constexpr int kPartStride = 6144;  // floats per partial: the gradient, then the loss
+static_assert(NPAR < kPartStride, "partial gradient");
 struct GradSmem {
-    float P[NPAR];
-    float X[kRays][PIN + 1];
-    float H1[kRays][PH + 1];
-    float H2[kRays][PH + 1];
-    float DZ[kRays][PO];
-    float DH2[kRays][PH + 1];
-    float DH1[kRays][PH + 1];
-    float loss[kRays];
+    float P[(NPAR + 3) / 4 * 4];
+    float X[PIN][kGLd];
+    float H1[PH][kGLd];
+    float H2[PH][kGLd];
+    float D1[PH][kGLd];
+    float D2[PH][kGLd];
+    float Z[PO][kGLd];  // logits, then dL/dz
+    uint32_t ray[kGRays];
+    float loss[kGThreads / 32];
 };
 
-// Gradient of the mean cross-entropy over a batch of B rays (B may span CTAs):
-// ray indices come from `idx` (when non-NULL) or from the counter-based hash.
-__global__ void __launch_bounds__(kRays) k_prop_grad(const float* __restrict__ params, const float* __restrict__ ro,
-                                                     const float* __restrict__ rd, const float2* __restrict__ root,
-                                                     const float* __restrict__ targets, uint32_t n, uint32_t B,
-                                                     uint64_t seed, uint64_t step, float* __restrict__ grad,
-                                                     float* __restrict__ loss) {
+// What an earlier step wrote is read after grid_wait with loads that go to L2 (__ldcg): this
+// grid may have started before it was written.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// acc[i] += w * v[i] over the four rays of v.
+__device__ __forceinline__ void fma4(float w, const float4& v, float (&acc)[4]) {
+    acc[0] = fmaf(w, v.x, acc[0]);
+    acc[1] = fmaf(w, v.y, acc[1]);
+    acc[2] = fmaf(w, v.z, acc[2]);
+    acc[3] = fmaf(w, v.w, acc[3]);
+}
+__device__ __forceinline__ float dot4(const float4& a, const float4& b, float acc) {
+    return fmaf(a.w, b.w, fmaf(a.z, b.z, fmaf(a.y, b.y, fmaf(a.x, b.x, acc))));
+}
+__device__ __forceinline__ float4 row4(const float* row, int r) { return *reinterpret_cast<const float4*>(row + r); }
+
+__global__ void __launch_bounds__(kGThreads, 1) k_prop_grad(const float* __restrict__ params, const float* __restrict__ ro,
+                                                         const float* __restrict__ rd, const float2* __restrict__ root,
+                                                         const float* __restrict__ targets, uint32_t n, uint32_t B,
+                                                         uint64_t seed, uint64_t step, float* __restrict__ part) {
     extern __shared__ __align__(16) uint8_t smraw[];
     GradSmem& S = *reinterpret_cast<GradSmem*>(smraw);
-    for (int i = threadIdx.x; i < NPAR; i += blockDim.x) S.P[i] = params[i];
-    const uint32_t bi = blockIdx.x * kRays + threadIdx.x;
-    const bool valid = bi < B;
     const int t = threadIdx.x;
-    uint32_t r = 0;
-    float o[3] = {0.f, 0.f, 0.f}, d[3] = {1.f, 0.f, 0.f}, t0 = 0.f;
-    if (valid) {
-        r = B == n && seed == 0 ? bi : batch_ray(seed, step, bi, n);
+    grid_launch();
+    // this thread's outputs of the gradient contractions, summed over the CTA's tiles
+    float g1[2][3] = {}, g2[2] = {}, g3[5] = {}, gb = 0.0f, loss = 0.0f;
+    const int o1 = 2 * (t / 30), f1 = 3 * (t % 30);        // W1: rows o1, o1 + 1, columns f1 .. f1 + 2 (t < 480)
+    const int o2 = t >> 4, i2 = t & 15;                    // W2: row o2, columns i2, i2 + 16
+    const int b3 = 5 * (t >> 5), i3 = t & 31;              // W3: rows b3 .. b3 + 4, column i3 (t < 416)
+    const float* brow = t < PH ? S.D1[t] : (t < 2 * PH ? S.D2[t - PH] : S.Z[t < 2 * PH + PO ? t - 2 * PH : 0]);
+    const uint32_t n_tiles = (B + kGRays - 1) / kGRays;
+    bool first = true;
+    for (uint32_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+        if (!first) __syncthreads();  // the previous tile's contractions are done
+        {  // features: eight threads per ray, each every eighth sine / cosine pair
+            const int r = t & (kGRays - 1), part_ = t / kGRays;
+            const uint32_t bi = tile * kGRays + r;
+            const bool valid = bi < B;
+            float o[3] = {0.f, 0.f, 0.f}, d[3] = {1.f, 0.f, 0.f}, e[3], t0 = 0.f;
+            if (valid) {
+                const uint32_t ray = B == n && seed == 0 ? bi : batch_ray(seed, step, bi, n);
+                if (part_ == 0) S.ray[r] = ray;
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            o[a] = __ldg(ro + 3 * (size_t)r + a);
-            d[a] = __ldg(rd + 3 * (size_t)r + a);
+                for (int a = 0; a < 3; ++a) {
+                    o[a] = __ldg(ro + 3 * (size_t)ray + a);
+                    d[a] = __ldg(rd + 3 * (size_t)ray + a);
+                }
+                t0 = __ldg(&root[ray].x);
+            }
+#pragma unroll
+            for (int a = 0; a < 3; ++a) e[a] = __fadd_rn(o[a], __fmul_rn(t0, d[a]));
+            if (part_ == 0) {
+#pragma unroll
+                for (int a = 0; a < 3; ++a) {
+                    S.X[a][r] = e[a];
+                    S.X[63 + a][r] = d[a];
+                }
+            }
+            for (int p = part_; p < 42; p += kGThreads / kGRays) {
+                const int k = p < 30 ? p / 3 : (p - 30) / 3, a = p % 3;
+                const float v = p < 30 ? (a == 0 ? e[0] : (a == 1 ? e[1] : e[2])) : (a == 0 ? d[0] : (a == 1 ? d[1] : d[2]));
+                const int f = (p < 30 ? 3 : 66) + 6 * k + a;
+                sincospif(v * (float)(1 << k), &S.X[f][r], &S.X[f + 3][r]);
+            }
         }
-        t0 = root[r].x;
-    }
-    prop_features<1>(o, d, t0, S.X[t]);
-    __syncthreads();
-    float h1[PH], h2[PH], q[PO];
-    prop_forward(S.P, S.X[t], h1, h2, q);
-    float L = 0.0f;
-    if (valid) {
-        float ps = 0.0f;
-#pragma unroll
-        for (int b = 0; b < PO; ++b) {
-            const float p = __ldg(targets + (size_t)r * PO + b);
-            if (p > 0.0f) L -= p * logf(q[b]);
-            ps += p;
-            S.DZ[t][b] = -p;
+        if (first) {
+            grid_wait();  // the previous step's parameters
+            for (int i = t; i < NPAR; i += kGThreads) S.P[i] = __ldcg(params + i);
+            first = false;
         }
+        __syncthreads();
+        // layers: four rays x one output per thread, accumulated from the bias over the
+        // inputs in order
+        const int r4 = 4 * (t & 15), o = t >> 4;
+        {
+            float acc[4];
+            acc[0] = acc[1] = acc[2] = acc[3] = S.P[OFF_B1 + o];
+#pragma unroll 6
+            for (int f = 0; f < PIN; ++f) fma4(S.P[OFF_W1 + o * PIN + f], row4(S.X[f], r4), acc);
+            *reinterpret_cast<float4*>(&S.H1[o][r4]) =
+                make_float4(fmaxf(acc[0], 0.f), fmaxf(acc[1], 0.f), fmaxf(acc[2], 0.f), fmaxf(acc[3], 0.f));
+        }
+        __syncthreads();
+        {
+            float acc[4];
+            acc[0] = acc[1] = acc[2] = acc[3] = S.P[OFF_B2 + o];
+#pragma unroll 8
+            for (int i = 0; i < PH; ++i) fma4(S.P[OFF_W2 + o * PH + i], row4(S.H1[i], r4), acc);
+            *reinterpret_cast<float4*>(&S.H2[o][r4]) =
+                make_float4(fmaxf(acc[0], 0.f), fmaxf(acc[1], 0.f), fmaxf(acc[2], 0.f), fmaxf(acc[3], 0.f));
+        }
+        __syncthreads();
+        for (int b = o; b < PO; b += PH) {
+            float acc[4];
+            acc[0] = acc[1] = acc[2] = acc[3] = S.P[OFF_B3 + b];
+#pragma unroll 8
+            for (int i = 0; i < PH; ++i) fma4(S.P[OFF_W3 + b * PH + i], row4(S.H2[i], r4), acc);
+            *reinterpret_cast<float4*>(&S.Z[b][r4]) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+        }
+        __syncthreads();
+        {  // softmax, loss and dL/dz: eight threads per ray
+            const int r = t >> 3, s = t & 7;
+            const bool valid = tile * kGRays + r < B;
+            float q[9], m = -INFINITY, sum = 0.0f, ps = 0.0f, p[9];
+            const float* tg = targets + (valid ? (size_t)S.ray[r] * PO : 0);
 #pragma unroll
-        for (int b = 0; b < PO; ++b) S.DZ[t][b] += q[b] * ps;  // dL/dz = q sum(p) - p
-    } else {
-        for (int b = 0; b < PO; ++b) S.DZ[t][b] = 0.0f;
+            for (int i = 0; i < 9; ++i) {
+                const int b = s + 8 * i;
+                const bool in = b < PO;
+                q[i] = in ? S.Z[b][r] : -INFINITY;
+                p[i] = in && valid ? __ldg(tg + b) : 0.0f;
+                m = fmaxf(m, q[i]);
+                ps += p[i];
+            }
+#pragma unroll
+            for (int w = 1; w < 8; w <<= 1) {
+                m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, w));
+                ps += __shfl_xor_sync(0xffffffffu, ps, w);
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                q[i] = s + 8 * i < PO ? expf(q[i] - m) : 0.0f;
+                sum += q[i];
+            }
+#pragma unroll
+            for (int w = 1; w < 8; w <<= 1) sum += __shfl_xor_sync(0xffffffffu, sum, w);
+            const float inv = 1.0f / sum;
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                const int b = s + 8 * i;
+                q[i] *= inv;
+                if (p[i] > 0.0f) loss -= p[i] * logf(q[i]);
+                if (b < PO) S.Z[b][r] = valid ? fmaf(q[i], ps, -p[i]) : 0.0f;  // q sum(p) - p
+            }
+        }
+        __syncthreads();
+        {  // back through layer 3 and the second ReLU
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 5
+            for (int b = 0; b < PO; ++b) fma4(S.P[OFF_W3 + b * PH + o], row4(S.Z[b], r4), acc);
+            const float4 h = row4(S.H2[o], r4);
+            *reinterpret_cast<float4*>(&S.D2[o][r4]) = make_float4(h.x > 0.f ? acc[0] : 0.f, h.y > 0.f ? acc[1] : 0.f,
+                                                                   h.z > 0.f ? acc[2] : 0.f, h.w > 0.f ? acc[3] : 0.f);
+        }
+        __syncthreads();
+        {  // ... layer 2 and the first
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll 8
+            for (int i = 0; i < PH; ++i) fma4(S.P[OFF_W2 + i * PH + o], row4(S.D2[i], r4), acc);
+            const float4 h = row4(S.H1[o], r4);
+            *reinterpret_cast<float4*>(&S.D1[o][r4]) = make_float4(h.x > 0.f ? acc[0] : 0.f, h.y > 0.f ? acc[1] : 0.f,
+                                                                   h.z > 0.f ? acc[2] : 0.f, h.w > 0.f ? acc[3] : 0.f);
+        }
+        __syncthreads();
+        // contractions over the tile's rays
+        if (t < 480) {
+#pragma unroll 2
+            for (int r = 0; r < kGRays; r += 4) {
+                const float4 a0 = row4(S.D1[o1], r), a1 = row4(S.D1[o1 + 1], r);
+#pragma unroll
+                for (int j = 0; j < 3; ++j) {
+                    const float4 x = row4(S.X[f1 + j], r);
+                    g1[0][j] = dot4(a0, x, g1[0][j]);
+                    g1[1][j] = dot4(a1, x, g1[1][j]);
+                }
+            }
+        }
+#pragma unroll 4
+        for (int r = 0; r < kGRays; r += 4) {
+            const float4 a = row4(S.D2[o2], r);
+            g2[0] = dot4(a, row4(S.H1[i2], r), g2[0]);
+            g2[1] = dot4(a, row4(S.H1[i2 + 16], r), g2[1]);
+        }
+        if (t < 416) {
+#pragma unroll 2
+            for (int r = 0; r < kGRays; r += 4) {
+                const float4 h = row4(S.H2[i3], r);
+#pragma unroll
+                for (int j = 0; j < 5; ++j) g3[j] = dot4(row4(S.Z[b3 + j], r), h, g3[j]);
+            }
+        }
+        if (t < 2 * PH + PO) {
+#pragma unroll 4
+            for (int r = 0; r < kGRays; r += 4) {
+                const float4 a = row4(brow, r);
+                gb = gb + a.x + a.y + a.z + a.w;
+            }
+        }
     }
-    S.loss[t] = L;
-#pragma unroll
-    for (int i = 0; i < PH; ++i) {
-        S.H1[t][i] = h1[i];
-        S.H2[t][i] = h2[i];
-    }
-    // back through layer 3 and the second ReLU, then layer 2 and the first ReLU
-    float dh2[PH];
-#pragma unroll
-    for (int i = 0; i < PH; ++i) {
-        float acc = 0.0f;
-        for (int b = 0; b < PO; ++b) acc = fmaf(S.P[OFF_W3 + b * PH + i], S.DZ[t][b], acc);
-        dh2[i] = h2[i] > 0.0f ? acc : 0.0f;
-        S.DH2[t][i] = dh2[i];
-    }
-#pragma unroll
-    for (int i = 0; i < PH; ++i) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int o2 = 0; o2 < PH; ++o2) acc = fmaf(S.P[OFF_W2 + o2 * PH + i], dh2[o2], acc);
-        S.DH1[t][i] = h1[i] > 0.0f ? acc : 0.0f;
-    }
-    __syncthreads();
-    // gradient contractions over this CTA's rays, scaled by 1 / B (mean loss)
+    // this CTA's partial, scaled by 1 / B (mean loss)
     const float sc = 1.0f / (float)B;
-    for (int e = threadIdx.x; e < NPAR; e += blockDim.x) {
-        float acc = 0.0f;
-        if (e < OFF_B1) {  // W1[o][f]: sum_r DH1[r][o] X[r][f]
-            const int o1 = e / PIN, f = e - o1 * PIN;
-            for (int rr = 0; rr < kRays; ++rr) acc = fmaf(S.DH1[rr][o1], S.X[rr][f], acc);
-        } else if (e < OFF_W2) {
-            const int o1 = e - OFF_B1;
-            for (int rr = 0; rr < kRays; ++rr) acc += S.DH1[rr][o1];
-        } else if (e < OFF_B2) {
-            const int k = e - OFF_W2, o2 = k / PH, i = k - o2 * PH;
-            for (int rr = 0; rr < kRays; ++rr) acc = fmaf(S.DH2[rr][o2], S.H1[rr][i], acc);
-        } else if (e < OFF_W3) {
-            const int o2 = e - OFF_B2;
-            for (int rr = 0; rr < kRays; ++rr) acc += S.DH2[rr][o2];
-        } else if (e < OFF_B3) {
-            const int k = e - OFF_W3, b = k / PH, i = k - b * PH;
-            for (int rr = 0; rr < kRays; ++rr) acc = fmaf(S.DZ[rr][b], S.H2[rr][i], acc);
-        } else {
-            const int b = e - OFF_B3;
-            for (int rr = 0; rr < kRays; ++rr) acc += S.DZ[rr][b];
-        }
-        atomicAdd(grad + e, acc * sc);
-    }
-    if (threadIdx.x < 32) {
-        float l = 0.0f;
-        for (int rr = threadIdx.x; rr < kRays; rr += 32) l += S.loss[rr];
+    float* out = part + (size_t)blockIdx.x * kPartStride;
+    if (t < 480) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-        if (threadIdx.x == 0) atomicAdd(loss, l * sc);
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) out[OFF_W1 + (o1 + i) * PIN + f1 + j] = g1[i][j] * sc;
+    }
+    out[OFF_W2 + o2 * PH + i2] = g2[0] * sc;
+    out[OFF_W2 + o2 * PH + i2 + 16] = g2[1] * sc;
+    if (t < 416) {
+#pragma unroll
+        for (int j = 0; j < 5; ++j) out[OFF_W3 + (b3 + j) * PH + i3] = g3[j] * sc;
+    }
+    if (t < 2 * PH + PO)
+        out[(t < PH ? OFF_B1 + t : (t < 2 * PH ? OFF_B2 + t - PH : OFF_B3 + t - 2 * PH))] = gb * sc;
+#pragma unroll
+    for (int w = 16; w > 0; w >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, w);
+    if ((t & 31) == 0) S.loss[t >> 5] = loss;
+    __syncthreads();
+    if (t == 0) {
+        float l = 0.0f;
+#pragma unroll
+        for (int i = 0; i < kGThreads / 32; ++i) l += S.loss[i];
+        out[NPAR] = l * sc;
     }
 }
 
-// Adam (Kingma and Ba) with bias correction; t counts from 1.  Clears the gradient.
-__global__ void k_prop_adam(float* __restrict__ P, float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, int t, float lr, float b1, float b2, float eps) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+// Sums the partial gradients (eight warps take every eighth CTA's, in order) and, with P,
+// applies Adam (Kingma and Ba) with bias correction, t counting from 1; without, stores the
+// gradient.  One parameter per lane; the value after the last parameter is the loss.
+__global__ void __launch_bounds__(256) k_prop_reduce(const float* __restrict__ part, int n_part, float* __restrict__ P,
+                                                     float* __restrict__ m, float* __restrict__ v, int t, float lr,
+                                                     float b1, float b2, float eps, float* __restrict__ grad,
+                                                     float* __restrict__ loss) {
+    __shared__ float s[8][32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int i = blockIdx.x * 32 + lane;
+    grid_launch();
+    grid_wait();
+    float a = 0.0f;
+#pragma unroll 16
+    for (int c = w; c < n_part; c += 8) a += __ldcg(part + (size_t)c * kPartStride + i);
+    s[w][lane] = a;
+    __syncthreads();
+    if (w) return;
+    float gi = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) gi += s[k][lane];
+    if (i == NPAR) *loss = gi;
     if (i >= NPAR) return;
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.0f - b1) * gi;
-    const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
+    if (!P) {
+        grad[i] = gi;
+        return;
+    }
+    const float mi = b1 * __ldcg(m + i) + (1.0f - b1) * gi;
+    const float vi = b2 * __ldcg(v + i) + (1.0f - b2) * gi * gi;
     m[i] = mi;
     v[i] = vi;
     const float c1 = 1.0f - powf(b1, (float)t), c2 = 1.0f - powf(b2, (float)t);
-    P[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    g[i] = 0.0f;
+    P[i] = __ldcg(P + i) - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+}
+constexpr int kReduceBlocks = (NPAR + 1 + 31) / 32;
+static_assert(kReduceBlocks * 32 <= kPartStride, "the last block stays inside a partial");
+
+// A launch that may start before its predecessor in the stream has ended (pdl; the kernel
+// then waits for it itself), or an ordinary one.
+template <class... Args>
+cudaError_t launch_after(cudaStream_t s, bool pdl, void (*kern)(Args...), unsigned grid, unsigned threads, size_t smem,
+                         Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
 }  // namespace
@@ -774,18 +949,22 @@ cudaError_t prepare_proposal(int* infer_grid) {
     return cudaFuncSetAttribute(k_prop_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
 }
 
-cudaError_t launch_prop_grad(cudaStream_t s, const float* params, const float* ro, const float* rd,
-                             const float2* root, const float* targets, uint32_t n, uint32_t batch, uint64_t seed,
-                             uint64_t step, float* grad, float* loss) {
-    if (batch == 0) return cudaSuccess;
-    k_prop_grad<<<(batch + kRays - 1) / kRays, kRays, sizeof(GradSmem), s>>>(params, ro, rd, root, targets, n, batch,
-                                                                            seed, step, grad, loss);
-    return cudaGetLastError();
-}
+size_t prop_partial_floats() { return (size_t)kPartCtas * kPartStride; }
 
-cudaError_t launch_prop_adam(cudaStream_t s, float* P, float* g, float* m, float* v, int t, float lr) {
-    k_prop_adam<<<(NPAR + 255) / 256, 256, 0, s>>>(P, g, m, v, t, lr, 0.9f, 0.999f, 1e-8f);
-    return cudaGetLastError();
+cudaError_t launch_prop_step(cudaStream_t s, bool first, const float* params, const float* ro, const float* rd,
+                             const float2* root, const float* targets, uint32_t n, uint32_t batch, uint64_t seed,
+                             uint64_t step, float* part, float* P, float* m, float* v, float lr, float* grad,
+                             float* loss) {
+    if (batch == 0) return cudaSuccess;
+    const uint32_t tiles = (batch + kGRays - 1) / kGRays;
+    const unsigned grid = tiles < (uint32_t)kPartCtas ? tiles : (unsigned)kPartCtas;
+    // the first launch of a call is an ordinary one: what it reads may be the stream's
+    // latest work; every later launch waits for its predecessor in the kernel
+    const cudaError_t e = launch_after(s, !first, k_prop_grad, grid, kGThreads, sizeof(GradSmem), params, ro, rd, root,
+                                       targets, n, batch, seed, step, part);
+    if (e != cudaSuccess) return e;
+    return launch_after(s, true, k_prop_reduce, (unsigned)kReduceBlocks, 256u, (size_t)0, (const float*)part, (int)grid,
+                        P, m, v, (int)step, lr, 0.9f, 0.999f, 1e-8f, grad, loss);
 }
 
 }  // namespace amnerf

@@ -99,8 +99,10 @@ cudaError_t launch_traverse(cudaStream_t s, const float* ro, const float* rd, ui
 // acc (may be NULL) accumulates (crossings, tiles) over the waves of one render.
 cudaError_t launch_scan(cudaStream_t s, const uint32_t* counts, int n_leaves, int cpt, uint32_t* offsets,
                         uint32_t* tile_off, uint32_t* cursor, uint64_t* stats, uint64_t* acc = nullptr);
-cudaError_t launch_scatter(cudaStream_t s, const uint8_t* n_x, const uint16_t* xleaf, uint32_t n_rays, int maxc,
-                           uint32_t* cursor, uint32_t* order, int n_leaves);
+// Both for a whole batch (one launch when it is small).  cursor: zero on entry.
+cudaError_t launch_group(cudaStream_t s, const uint8_t* n_x, const uint16_t* xleaf, uint32_t n_rays, int maxc,
+                         const uint32_t* counts, int n_leaves, int cpt, uint32_t* offsets, uint32_t* tile_off,
+                         uint32_t* cursor, uint64_t* stats, uint32_t* order);
 // One wave: crossing k of ray r takes part when k_lo <= k < min(n_x[r], k_hi) and
 // alive[r] (alive == NULL: every ray).  count: only the per-leaf totals, added to
 // cursor (zeroed by the caller); else the grouped scatter from the scanned cursor.

@@ -15,6 +15,8 @@
 using namespace amnerf;
 
 constexpr int kStatSlots = 10;  // device statistics words (see amnerf_ctx::d_stats)
+constexpr size_t kZeroBytes = kRayCounterBytes * 2 + 256;  // in front of the network counts
+static_assert(kStatSlots * sizeof(uint64_t) <= 256, "statistics words");
 constexpr int kDefaultWidthSplit = 1;  // BF16 hidden-width tiling when the caller sets none
 
 struct amnerf_ctx {
@@ -40,11 +42,14 @@ struct amnerf_ctx {
     size_t leaf_stride = 0;  // bytes
     void* d_weights = nullptr;
     void* d_split = nullptr;  // FP32 networks: their split operands (tensor-core path; null: SIMT only)
+    // ray counters | statistics | network counts | cursors, zeroed together at the start of a
+    // render
+    uint8_t* d_zero = nullptr;
     // per-network scratch (sized for kMaxNets)
-    uint32_t* d_counts = nullptr;
+    uint32_t* d_counts = nullptr;  // in d_zero
     uint32_t* d_offsets = nullptr;
     uint32_t* d_tile_off = nullptr;
-    uint32_t* d_cursor = nullptr;
+    uint32_t* d_cursor = nullptr;  // in d_zero
     // [0] crossings [1] tiles [2] composited [3] fallback rays [4] [5] one wave's
     // crossings and tiles [6] dynamic tile counter [8] [9] crossings and tiles over waves
     uint64_t* d_stats = nullptr;
@@ -289,17 +294,18 @@ amnerf_status amnerf_create(amnerf_ctx** out, int device, void* cuda_stream) {
     if ((e = cudaSetDevice(device)) != cudaSuccess ||
         (e = prepare_group()) != cudaSuccess ||
         (e = prepare_traverse()) != cudaSuccess ||
-        (e = cudaMalloc((void**)&ctx->d_counts, sizeof(uint32_t) * kMaxNets)) != cudaSuccess ||
+        (e = cudaMalloc((void**)&ctx->d_zero, kZeroBytes + 2 * sizeof(uint32_t) * kMaxNets)) != cudaSuccess ||
         (e = cudaMalloc((void**)&ctx->d_offsets, sizeof(uint32_t) * (kMaxNets + 1))) != cudaSuccess ||
         (e = cudaMalloc((void**)&ctx->d_tile_off, sizeof(uint32_t) * (kMaxNets + 1))) != cudaSuccess ||
-        (e = cudaMalloc((void**)&ctx->d_cursor, sizeof(uint32_t) * kMaxNets)) != cudaSuccess ||
-        (e = cudaMalloc((void**)&ctx->d_stats, sizeof(uint64_t) * kStatSlots)) != cudaSuccess ||
-        (e = cudaMalloc((void**)&ctx->d_ray_ctr, kRayCounterBytes * 2)) != cudaSuccess ||
         (e = cudaMalloc((void**)&ctx->d_err, sizeof(int))) != cudaSuccess ||
         (e = cudaMemset(ctx->d_err, 0, sizeof(int))) != cudaSuccess) {
         amnerf_destroy(ctx);
         return e == cudaErrorMemoryAllocation ? AMNERF_E_NOMEM : AMNERF_E_CUDA;
     }
+    ctx->d_ray_ctr = reinterpret_cast<uint32_t*>(ctx->d_zero);
+    ctx->d_stats = reinterpret_cast<uint64_t*>(ctx->d_zero + kRayCounterBytes * 2);
+    ctx->d_counts = reinterpret_cast<uint32_t*>(ctx->d_zero + kZeroBytes);
+    ctx->d_cursor = ctx->d_counts + kMaxNets;  // a render puts it right behind its counts
     for (int i = 0; i < 6; ++i) cudaEventCreate(&ctx->ev[i]);
     *out = ctx;
     return AMNERF_OK;
@@ -330,12 +336,9 @@ void amnerf_destroy(amnerf_ctx* ctx) {
     dfree(ctx->d_weights);
     dfree(ctx->d_split);
     dfree(ctx->d_amax);
-    dfree(ctx->d_counts);
+    dfree(ctx->d_zero);
     dfree(ctx->d_offsets);
     dfree(ctx->d_tile_off);
-    dfree(ctx->d_cursor);
-    dfree(ctx->d_stats);
-    dfree(ctx->d_ray_ctr);
     dfree(ctx->d_err);
     dfree(ctx->d_hbuf);
     dfree(ctx->d_prop);
@@ -560,9 +563,9 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
     hier.lod = p->lod;
     hier.node_net = ctx->d_node_net;
     if (ctx->timing) cudaEventRecord(ctx->ev[0], s);
-    CK(cudaMemsetAsync(ctx->d_counts, 0, sizeof(uint32_t) * L, s), "memset");
-    CK(cudaMemsetAsync(ctx->d_stats, 0, sizeof(uint64_t) * kStatSlots, s), "memset");
-    CK(cudaMemsetAsync(ctx->d_ray_ctr, 0, kRayCounterBytes * 2, s), "memset");
+    // ray counters, statistics, the L counts and the L cursors lie together: one memset
+    ctx->d_cursor = ctx->d_counts + L;
+    CK(cudaMemsetAsync(ctx->d_zero, 0, kZeroBytes + 2 * sizeof(uint32_t) * L, s), "memset");
     const uint64_t* mask = nullptr;
     const uint8_t* fallback = nullptr;
     if (p->use_proposal && n > 0) {
@@ -603,18 +606,20 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
            "traverse launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[1], s);
-    CK(launch_scan(s, ctx->d_counts, L, kTileRows / steps, ctx->d_offsets, ctx->d_tile_off, ctx->d_cursor,
-                   ctx->d_stats),
-       "scan launch");
     // waves: the rays' crossings in groups of ert_wave, each group only for the rays
     // that have not terminated, so that samples behind an opaque crossing are never
     // evaluated (the number of waves depends only on maxc: no host synchronisation)
     const bool waves = p->ert_wave > 0 && n > 0 && !bins_out;
     if (waves) {
+        CK(launch_scan(s, ctx->d_counts, L, kTileRows / steps, ctx->d_offsets, ctx->d_tile_off, ctx->d_cursor,
+                       ctx->d_stats),
+           "scan launch");
         st = ensure_wave_scratch(ctx, (size_t)n);
         if (st != AMNERF_OK) return st;
     } else {
-        CK(launch_scatter(s, ctx->d_nx, ctx->d_xleaf, nn, maxc, ctx->d_cursor, ctx->d_order, L), "scatter launch");
+        CK(launch_group(s, ctx->d_nx, ctx->d_xleaf, nn, maxc, ctx->d_counts, L, kTileRows / steps, ctx->d_offsets,
+                        ctx->d_tile_off, ctx->d_cursor, ctx->d_stats, ctx->d_order),
+           "grouping launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[2], s);
     // the network over the grouped crossings whose per-wave counts (crossings, tiles)

@@ -90,6 +90,12 @@ __device__ __forceinline__ void load_crossing_now(const void* __restrict__ slot_
     }
 }
 
+__device__ __forceinline__ float2 load_interval_now(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+
 template <bool HALF>
 __device__ __forceinline__ float4 slot_value(const RawSlot<HALF>& r) {
     if constexpr (HALF) {
@@ -335,15 +341,21 @@ __global__ void __launch_bounds__(256) k_composite_lane(
         const float2* xr = xing + (size_t)ray * maxc;
         const size_t row = (size_t)ray * cap;
         bool alive = true;
-        // crossing k + 1's slots are loaded while crossing k is composited
+        // crossing k + 1's slots and interval are loaded while crossing k is composited (two or
+        // three ahead were no faster: 626 us at 5.1 M rays with one, 672 and 686)
         RawSlot<HALF> vn[kSteps];
-        if (k_lo < nx) load_crossing_now<HALF, kSteps>(slot_out, row + (size_t)(k_lo * kSteps), vn);
+        float2 xn = make_float2(0.f, 0.f);
+        auto load_next = [&](int k) {
+            load_crossing_now<HALF, kSteps>(slot_out, row + (size_t)(k * kSteps), vn);
+            xn = load_interval_now(xr + k);
+        };
+        if (k_lo < nx) load_next(k_lo);
         for (int k = k_lo; k < nx && alive; ++k) {
-            const float2 x = __ldg(xr + k);
+            const float2 x = xn;
             RawSlot<HALF> v[kSteps];
 #pragma unroll
             for (int j = 0; j < kSteps; ++j) v[j] = vn[j];
-            if (k + 1 < nx) load_crossing_now<HALF, kSteps>(slot_out, row + (size_t)((k + 1) * kSteps), vn);
+            if (k + 1 < nx) load_next(k + 1);
             // same FP32 operations as the sampling step: delta = (t_out - t_in) / steps
             // (exact: a power of two), t_j = t_in + (j + 1/2) delta
             const float delta = __fmul_rn(__fsub_rn(x.y, x.x), 1.0f / kSteps);

@@ -20,22 +20,26 @@
 // (256 networks of 4 x 64), 2.6e-7 and 7.0e-7 against 2.5e-7 and 2.7e-7 with weights three
 // times as large; the largest single error is lower in every scene and shape measured.
 //
-// What bounds it: a 4 x 64 tile takes 135 MMAs, about 4 300 cycles of the tensor pipe, and
-// its rows about 3 000 instruction issues per SM sub-partition (42 sincospif per row, nine
-// instructions per split pair); three tiles of 168 TMEM columns are in flight per SM.  One
-// 800 x 800 view, network step: 7.6 ms (the SIMT kernel 37.6 ms, 46 % of the FP32 lanes'
-// peak); tensor pipe 52 %, issue 54 %.
+// What bounds it: a 4 x 64 tile takes 135 MMAs, about 4 400 cycles of the tensor pipe, and
+// its rows about 2 500 instruction issues per SM sub-partition (nine instructions per split
+// pair, 30 per sincospif); three tiles of 168 TMEM columns are in flight per SM, each
+// alternating between the two.  One 800 x 800 view (300 k tiles), network step: SIMT kernel
+// 37.6 ms (46 % of the FP32 lanes' peak); one thread per row 7.4 ms; two threads per row
+// (each half of a chunk's columns, half of an accumulator row) 7.1; with the staging in a
+// warp of its own, out of the issuing warps, 6.5 ms.
 //
-// Structure, as k_mlp_tc: compute warpgroups of 128 threads, one thread per sample row
-// (TMEM lane), and one auxiliary warp per group that stages the crossings, loads weights
-// and issues the MMAs.  A network's split weights take three times a BF16 network's (123 KB
-// at 4 x 64), so the groups of a CTA share one copy: the CTA's contiguous range of tiles is
-// cut at leaf changes, its groups take a leaf's tiles in turn, and at a leaf change the
-// auxiliary warps meet on an mbarrier before one of them loads the next leaf's weights.
-// Layer 0's 96 input columns (90 features, the constant 1 of the bias, padding) are written
-// in three chunks of 32 (kPerm): all three h parts stay in TMEM for the last products, the
-// m and l parts of a chunk share one buffer.  While the head runs, a group encodes the
-// first chunk of its next tile.  Every wait is bounded.
+// Structure, as k_mlp_tc: per tile in flight two compute warpgroups, whose threads r and
+// r + 128 own sample row (TMEM lane) r, and one auxiliary warp that loads weights and issues
+// the MMAs; one more warp stages the crossings of all groups.  A network's split weights
+// take three times a BF16 network's (123 KB at 4 x 64), so the groups of a CTA share one
+// copy: the CTA's contiguous range of tiles is cut at leaf changes, its groups take a
+// leaf's tiles in turn, and at a leaf change the auxiliary warps meet on an mbarrier before
+// one of them loads the next leaf's weights.  Layer 0's 96 input columns (90 features, the
+// constant 1 of the bias, padding) are written in three chunks of 32 (kPerm): all three h
+// parts stay in TMEM for the last products, the m and l parts of a chunk share one buffer.
+// The samples of a crossing share their direction's features (eight lanes compute a pair
+// each and exchange them, at 8 samples per crossing or more).  While the head runs, a group
+// encodes the first chunk of its next tile.  Every wait is bounded.
 //
 // Kept on the SIMT kernel: calibration (per-layer input maxima), other encodings than
 // lx = 10, ld = 4, and networks whose split weights do not fit the shared memory.
@@ -52,7 +56,9 @@ namespace {
 using namespace tcx;
 
 constexpr int kIn = 90, kInP = 96;  // encoded features; layer 0's K (bias at column 90)
-constexpr int kGroups = 3;          // compute warpgroups per CTA
+constexpr int kGroups = 3;          // tiles in flight per CTA, 256 threads (two per sample row) each
+constexpr int kTPR = 2;             // threads per row
+constexpr int kThreads = 128 * (kGroups * kTPR + 1);
 constexpr int kBiasK = 16;
 
 // TMEM columns of a group: D (accumulator), A (input parts), the constant ones of the bias
@@ -61,10 +67,6 @@ constexpr int kBiasK = 16;
 constexpr uint32_t kCols = 168, kA = 64, kOnes = 160;
 constexpr uint32_t kM0 = 48, kL0 = 64;
 static_assert(kGroups * kCols <= 512, "TMEM");
-
-// Registers per thread: 512 threads are launched with 128 each.
-constexpr int kComputeRegs = 144, kAuxRegs = 80;
-static_assert(kGroups * kComputeRegs + kAuxRegs <= (kGroups + 1) * 128, "the split draws on the launch's registers");
 
 // Layer 0's column order: column 2 i + 6 (and the next) hold sin and cos of pair i < 42
 // (octave i / 3 of coordinate i % 3 of x, the last 12 of d), columns 0..5 x and d.  Returns
@@ -100,9 +102,10 @@ struct SplitLayout {
 struct SplitShared {
     uint64_t bar_w;             // a leaf's weights
     uint64_t bar_seg;           // the groups are done with a leaf's weights
-    uint64_t bar_a[kGroups];    // input parts written by the four compute warps
+    uint64_t bar_a[kGroups];    // input parts written by the eight compute warps
     uint64_t bar_m[kGroups];    // MMAs completed
     uint64_t bar_s[kGroups];    // crossings staged
+    uint64_t bar_f[kGroups];    // a tile's staged crossings read by the eight compute warps
     int leaf[kGroups][kIdSlots];
     uint32_t tmem_base;
 };
@@ -182,20 +185,23 @@ __global__ void k_split_pack(const float* __restrict__ simt, size_t simt_stride,
 
 // HC > 0: the number of hidden layers fixed at compile time.
 template <int W, int HC, bool JIT>
-__global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g) {
+__global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
     const int hidden = HC > 0 ? HC : g.hidden;
     extern __shared__ __align__(1024) uint8_t smem[];
     const SplitLayout lay(W, hidden);
     SplitShared* sh = reinterpret_cast<SplitShared*>(smem + lay.stride);
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0);  // uniform for the compiler
-    const int q = warp & 3, tig = threadIdx.x & 127, lane_id = threadIdx.x & 31;
+    const int q = warp & 3, lane_id = threadIdx.x & 31;
+    const int row = 32 * q + lane_id;  // sample row = TMEM lane (two threads: half 0 and 1)
+    const int half = (warp >> 2) & 1;
     if (threadIdx.x == 0) {
         mbar_init(smem_u32(&sh->bar_w), 1);
         mbar_init(smem_u32(&sh->bar_seg), kGroups);
         for (int i = 0; i < kGroups; ++i) {
-            mbar_init(smem_u32(&sh->bar_a[i]), 4);
+            mbar_init(smem_u32(&sh->bar_a[i]), 4 * kTPR);
             mbar_init(smem_u32(&sh->bar_m[i]), 1);
             mbar_init(smem_u32(&sh->bar_s[i]), kStageArrivals);
+            mbar_init(smem_u32(&sh->bar_f[i]), 4 * kTPR);
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_proxy_async();
@@ -211,12 +217,13 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
 
-    const bool aux = warp >= 4 * kGroups;
-    const int gi = aux ? q : warp >> 2;  // this warp's group (aux: warp i of the last warpgroup serves group i)
+    const bool aux = warp >= 4 * kGroups * kTPR;
+    const int gi = aux ? q : warp >> 3;  // this warp's group (aux: warp i of the last warpgroup serves group i)
     const int gc = gi < kGroups ? gi : 0;
     const uint32_t bar_a = smem_u32(&sh->bar_a[gc]);
     const uint32_t bar_m = smem_u32(&sh->bar_m[gc]);
     const uint32_t bar_s = smem_u32(&sh->bar_s[gc]);
+    const uint32_t bar_f = smem_u32(&sh->bar_f[gc]);
     const uint32_t d_col = tmem + kCols * (uint32_t)gc;
     const uint32_t a_col = d_col + kA;
     const int cpt = kTileRows >> g.lg_steps;
@@ -236,7 +243,6 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
     const uint32_t t1 = min(t0 + per, t_end);
 
     if (aux) {
-        setmaxnreg_dec<kAuxRegs>();
         if (gi < kGroups) {
             const uint32_t w_addr = smem_u32(smem);
             const uint32_t bar_w = smem_u32(&sh->bar_w), bar_seg = smem_u32(&sh->bar_seg);
@@ -247,14 +253,7 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
             const uint32_t p0 = (uint32_t)(lay.part0() >> 4), ph_ = (uint32_t)(lay.parth() >> 4),
                            po = (uint32_t)(lay.parto() >> 4);
             const uint32_t idd = idesc_bf16(W), idh = idesc_bf16(16);
-            Stager st(g, stage, sh->leaf[gc], bar_s, cpt, t0 + (uint32_t)gi, kGroups, t1);
             uint32_t ph_a = 0, ph_w = 0, ph_seg = 0, n_m = 0;  // n_m: phases of bar_m committed
-            for (uint32_t n = 0; n < 3; ++n) st.ids(n);
-            cp_async_wait_all();
-            __syncwarp();
-            st.data(0);
-            st.data(1);
-            st.publish();
             uint32_t n = 0;
             // the leaves of the CTA's range in order, each with its tiles of this group
             uint32_t t = t0;
@@ -325,32 +324,70 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
                         for (int s = 0; s < W / 16; ++s) mma_bf16_ts_warp(d_col, a_col + 8u * s, b0 + 16u * s, id, 1u);
                         mma_commit_warp(bar_m);
                         ++n_m;
-                        // the slots' previous contents were read a tile ago; the arrival awaited
-                        // above follows the compute warps' wait for the phase before this one
-                        if (l == 1) {
-                            cp_async_wait_all();
-                            __syncwarp();
-                            st.data(n + 2);
-                            st.publish();
-                        }
-                        if (l == (hidden > 1 ? 2 : 1)) st.ids(n + 3);
                     }
                 }
                 t = seg_end;
                 if (t < t1) leaf = leaf_of_tile_warp(g.tile_off, leaf + 1, g.n_leaves, t);
             }
-            cp_async_wait_all();  // none in flight when the CTA ends
             if (!ok && lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
+        } else {
+            // the last warp stages every group's crossings: ids three tiles, intervals and rays
+            // two tiles ahead of what the group reads
+            auto group = [&](int i) {
+                return Stager(g, reinterpret_cast<uint8_t*>(sh) + kShBytes + i * stage_bytes(cpt), sh->leaf[i],
+                              smem_u32(&sh->bar_s[i]), cpt, t0 + (uint32_t)i, kGroups, t1);
+            };
+            Stager st[kGroups] = {group(0), group(1), group(2)};
+            uint32_t k[kGroups], last[kGroups];  // tiles whose reading is awaited next, and in all
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i) {
+                k[i] = 0;
+                last[i] = t0 + (uint32_t)i < t1 ? (t1 - t0 - (uint32_t)i + kGroups - 1) / kGroups : 0u;
+                for (uint32_t n = 0; n < 3; ++n) st[i].ids(n);
+            }
+            cp_async_wait_all();
+            __syncwarp();
+#pragma unroll
+            for (int i = 0; i < kGroups; ++i) {
+                st[i].data(0);
+                st[i].data(1);
+                st[i].publish();
+            }
+            // tile k's crossings read (and with them phase k awaited): tile k + 2's may take
+            // their slot, and be published as phase k + 1
+            unsigned long long since = clock64();
+            while (k[0] < last[0] || k[1] < last[1] || k[2] < last[2]) {
+                bool any = false;
+#pragma unroll
+                for (int i = 0; i < kGroups; ++i) {
+                    if (k[i] < last[i] && __all_sync(0xffffffffu, mbar_test(smem_u32(&sh->bar_f[i]), k[i] & 1u))) {
+                        cp_async_wait_all();  // tile k + 2's ids, copied a tile ago
+                        __syncwarp();
+                        st[i].data(k[i] + 2);
+                        st[i].publish();
+                        st[i].ids(k[i] + 3);
+                        ++k[i];
+                        any = true;
+                    }
+                }
+                const unsigned long long now = clock64();
+                if (any) since = now;
+                if (!__all_sync(0xffffffffu, now - since <= kWaitCycles)) {
+                    if (lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
+                    break;
+                }
+            }
+            cp_async_wait_all();  // none in flight when the CTA ends
         }
     } else {
-        setmaxnreg_inc<kComputeRegs>();
         const uint32_t lane = (uint32_t)(32 * q) << 16;
         const uint32_t d_row = d_col + lane, a_row = a_col + lane;
-        {
+        if (half == 0) {
             const uint32_t c8[8] = {0u, 0u, 0u, 0u, 0u, pack_bf16(1.0f, 1.0f), pack_bf16(1.0f, 0.0f), 0u};
             tmem_st8(d_row + kOnes, c8);
         }
-        const int ci = tig >> g.lg_steps, j = tig - (ci << g.lg_steps);
+        const int ci = row >> g.lg_steps, j = row - (ci << g.lg_steps);
+        const bool share = g.lg_steps >= 3;  // lanes 8 i .. 8 i + 7 belong to one crossing
         auto publish = [&]() {
             tmem_st_wait();
             tc_fence_before();
@@ -358,45 +395,76 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
             if (lane_id == 0) mbar_arrive(bar_a);
         };
         float x[3], d[3];
-        // chunk C of the layer-0 input: its split words
-        uint32_t wh[16], wm[16], wl[16];
-        auto encode = [&](auto chunk) {
-            constexpr int C = decltype(chunk)::value;
+        // this half's eight words (column pairs) of a chunk of the layer-0 input, split
+        uint32_t wh[8], wm[8], wl[8];
+        // pair p < 42: sine and cosine
+        auto pair = [&](int p, float& v0, float& v1) {
+            const int oct = p < 30 ? p / 3 : (p - 30) / 3;
+            sincospif((p < 30 ? x[p % 3] : d[p % 3]) * (float)(1 << oct), &v0, &v1);
+        };
+        auto encode_half = [&](auto chunk, auto hv) {
+            constexpr int C = decltype(chunk)::value, H = decltype(hv)::value;
+            constexpr int P0 = (32 * C + 16 * H - 6) / 2;  // pair of word 0 (chunk 0, half 0: from word 3)
+            constexpr int D0 = P0 < 30 ? 30 - P0 : 0;      // first word that holds a direction pair ...
+            constexpr int D1 = P0 + 8 < 42 ? 8 : 42 - P0;  // ... and one past the last
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                constexpr int kPairs = 42;
-                const int col = 32 * C + 2 * i;  // word i: columns col, col + 1
+            for (int i = 0; i < 8; ++i) {
+                const int col = 32 * C + 16 * H + 2 * i;
                 float v0, v1;
                 if (col < 6) {
                     v0 = col == 0 ? x[0] : (col == 2 ? x[2] : d[1]);
                     v1 = col == 0 ? x[1] : (col == 2 ? d[0] : d[2]);
-                } else {
-                    const int p = (col - 6) >> 1;
-                    if (p < kPairs) {
-                        const int oct = p < 30 ? p / 3 : (p - 30) / 3;
-                        sincospif((p < 30 ? x[p % 3] : d[p % 3]) * (float)(1 << oct), &v0, &v1);
-                    } else {  // the bias column's 1, then padding
-                        v0 = p == kPairs ? 1.0f : 0.0f;
-                        v1 = 0.0f;
-                    }
+                } else if (P0 + i < 42) {
+                    if (C == 2 && i >= D0 && share) continue;
+                    pair(P0 + i, v0, v1);
+                } else {  // the bias column's 1, then padding
+                    v0 = P0 + i == 42 ? 1.0f : 0.0f;
+                    v1 = 0.0f;
                 }
                 split3(v0, v1, wh[i], wm[i], wl[i]);
+            }
+            if (C == 2 && share) {
+                // the eight samples of a crossing share its direction: lane L of every eight
+                // computes word D0 + L, then all read them
+                const int p = min(P0 + D0 + (lane_id & 7), 41) - 30;
+                const int a = p % 3;
+                float v0, v1;
+                uint32_t h, m, l;
+                sincospif((a == 0 ? d[0] : (a == 1 ? d[1] : d[2])) * (float)(1 << (p / 3)), &v0, &v1);
+                split3(v0, v1, h, m, l);
+#pragma unroll
+                for (int i = D0; i < D1; ++i) {
+                    wh[i] = __shfl_sync(0xffffffffu, h, i - D0, 8);
+                    wm[i] = __shfl_sync(0xffffffffu, m, i - D0, 8);
+                    wl[i] = __shfl_sync(0xffffffffu, l, i - D0, 8);
+                }
             }
             pin(wh);
             pin(wm);
             pin(wl);
         };
+        auto encode = [&](auto chunk) {
+            if (half == 0) encode_half(chunk, std::integral_constant<int, 0>());
+            else encode_half(chunk, std::integral_constant<int, 1>());
+        };
         auto store = [&](int c) {
-            tmem_st16(a_row + 16u * c, wh);
-            tmem_st16(a_row + kM0, wm);
-            tmem_st16(a_row + kL0, wl);
+            tmem_st8(a_row + 16u * c + 8u * half, wh);
+            tmem_st8(a_row + kM0 + 8u * half, wm);
+            tmem_st8(a_row + kL0 + 8u * half, wl);
             publish();
         };
         float4 bo = make_float4(0.f, 0.f, 0.f, 0.f);
         uint32_t id = 0xffffffffu, ph_m = 0;
         int cur = -1;
+        // reads tile n's staged sample; phase n of bar_s (tile n + 1's crossings) has been awaited,
+        // so that the staging warp's next phase cannot be mistaken for it
+        auto place = [&](uint32_t n) {
+            id = staged_sample<JIT>(g, stage, cpt, n, ci, j, x, d);
+            __syncwarp();
+            if (lane_id == 0) mbar_arrive(bar_f);
+        };
         if (wait(bar_s, 0u) && leaf_s[0] >= 0) {
-            id = staged_sample<JIT>(g, stage, cpt, 0, ci, j, x, d);
+            place(0);
             encode(std::integral_constant<int, 0>());
             store(0);
         }
@@ -418,40 +486,46 @@ __global__ void __launch_bounds__(128 * (kGroups + 1), 1) k_mlp_split(MlpArgs g)
             ph_m ^= 1u;
             tc_fence_after();
             store(2);
-            if (n > 0 && !wait(bar_s, n & 1u)) break;  // tile n + 1's crossings
 #pragma unroll 1
             for (int l = 0; l < hidden; ++l) {
                 if (!wait(bar_m, ph_m)) break;
                 ph_m ^= 1u;
                 tc_fence_after();
-                // relu of the accumulator row, split, as the next layer's (or the head's) input
+                // relu of this half of the accumulator row, split, as the next layer's (or the
+                // head's) input, 16 columns at a time
 #pragma unroll
-                for (int h = 0; h < W / 32; ++h) {
-                    float v[32];
-                    tmem_ld32(d_row + 32u * h, v);
+                for (int i0 = 0; i0 < W / 32; ++i0) {
+                    const uint32_t col = (uint32_t)(W / 2) * half + 16u * i0;
+                    uint32_t v[16];
+                    tmem_ld16_nowait(d_row + col, v);
+                    tmem_ld_wait_regs(v);
 #pragma unroll
-                    for (int i = 0; i < 16; ++i)
-                        split3(fmaxf(v[2 * i], 0.0f), fmaxf(v[2 * i + 1], 0.0f), wh[i], wm[i], wl[i]);
-                    tmem_st16(a_row + 16u * h, wh);
-                    tmem_st16(a_row + 32u + 16u * h, wm);
-                    tmem_st16(a_row + 64u + 16u * h, wl);
+                    for (int i = 0; i < 8; ++i)
+                        split3(fmaxf(__uint_as_float(v[2 * i]), 0.0f), fmaxf(__uint_as_float(v[2 * i + 1]), 0.0f), wh[i],
+                               wm[i], wl[i]);
+                    tmem_st8(a_row + col / 2, wh);
+                    tmem_st8(a_row + 32u + col / 2, wm);
+                    tmem_st8(a_row + 64u + col / 2, wl);
                 }
                 publish();
             }
             if (!ok) break;
             // under the head: the next tile's sample and first chunk
             const uint32_t id_cur = id;
-            id = staged_sample<JIT>(g, stage, cpt, n + 1, ci, j, x, d);
+            if (!wait(bar_s, (n + 1) & 1u)) break;
+            place(n + 1);
             const bool more = leaf_s[(n + 1) & (kIdSlots - 1)] >= 0;
             encode(std::integral_constant<int, 0>());
             if (!wait(bar_m, ph_m)) break;
             ph_m ^= 1u;
             tc_fence_after();
             uint32_t z[4];
-            tmem_ld4_nowait(d_row, z);
-            tmem_ld_wait_regs(z);
+            if (half == 0) {
+                tmem_ld4_nowait(d_row, z);
+                tmem_ld_wait_regs(z);
+            }
             if (more) store(0);
-            if (id_cur != 0xffffffffu) {
+            if (half == 0 && id_cur != 0xffffffffu) {
                 float4 o;
                 o.x = softplus_f32(__uint_as_float(z[0]) + bo.x);
                 o.y = sigmoid_f32(__uint_as_float(z[1]) + bo.y);
@@ -487,13 +561,12 @@ cudaError_t prepare_w(int max_smem) {
 template <int W>
 cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid, size_t smem) {
     const bool hc = a.hidden == kHiddenFor<W>;
-    const int threads = 128 * (kGroups + 1);
     if (a.jitter) {
-        if (hc) k_mlp_split<W, kHiddenFor<W>, true><<<grid, threads, smem, s>>>(a);
-        else k_mlp_split<W, 0, true><<<grid, threads, smem, s>>>(a);
+        if (hc) k_mlp_split<W, kHiddenFor<W>, true><<<grid, kThreads, smem, s>>>(a);
+        else k_mlp_split<W, 0, true><<<grid, kThreads, smem, s>>>(a);
     } else {
-        if (hc) k_mlp_split<W, kHiddenFor<W>, false><<<grid, threads, smem, s>>>(a);
-        else k_mlp_split<W, 0, false><<<grid, threads, smem, s>>>(a);
+        if (hc) k_mlp_split<W, kHiddenFor<W>, false><<<grid, kThreads, smem, s>>>(a);
+        else k_mlp_split<W, 0, false><<<grid, kThreads, smem, s>>>(a);
     }
     return cudaGetLastError();
 }

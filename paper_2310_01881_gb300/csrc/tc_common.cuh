@@ -351,6 +351,13 @@ __device__ __forceinline__ void pin(uint32_t (&w)[N]) {
     for (int i = 0; i < N; ++i) asm volatile("" : "+r"(w[i]));
 }
 
+// max(a, b, c), a NaN ignored as by fmaxf.
+__device__ __forceinline__ float max3_f32(float a, float b, float c) {
+    float r;
+    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    return r;
+}
+
 // Head activations with the SFU exp/log/reciprocal (relative error ~1e-6, far below the
 // BF16/E4M3 operand rounding of this path).
 __device__ __forceinline__ float rcp_approx(float x) {

@@ -339,6 +339,15 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                 }
             }
             Stager st(g, stage, sh->leaf[gi], bar_s, cpt, t_next, t_step, t_stop);
+            // Tile n + 2's crossings.  A phase of bar_s may be published only when the compute
+            // warps have waited for the one before it (its parity would stand for both): that
+            // wait precedes their first arrival on bar_a in tile n, which must have been seen.
+            auto stage_next = [&](uint32_t n) {
+                cp_async_wait_all();
+                __syncwarp();
+                st.data(n + 2);
+                st.publish();
+            };
             uint32_t ph_w = 0, ph_h = 0, ph_a = 0;
             for (uint32_t n = 0; n < 3; ++n) st.ids(n);
             __syncwarp();
@@ -364,6 +373,10 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                         mma_bf16_ts_warp(d_col + kHeadCol, d_col + 8u * kk, desc_wo + 16u * kk, idd, 1u);
                     mma_commit_warp(bar_h);
                     if (leaf < 0) break;
+                    if (hidden == 1) {  // tile n - 1's only arrival has just been seen
+                        stage_next(n - 1);
+                        st.ids(n + 2);
+                    }
                     // the head reads D, which layer 0 overwrites, and its leaf's weights
                     if (!wait(bar_h, ph_h)) break;
                     ph_h ^= 1u;
@@ -427,13 +440,8 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                     // behind the later layers' issue, where the compute warps are in their
                     // epilogues: the slots' previous contents were read before tile n - 1's
                     // last layer, and tile n + 2's ids were copied a tile ago
-                    if (l == (hidden > 1 ? 1 : 0)) {
-                        cp_async_wait_all();
-                        __syncwarp();
-                        st.data(n + 2);
-                        st.publish();
-                    }
-                    if (l == (hidden > 2 ? 2 : hidden - 1)) st.ids(n + 3);
+                    if (hidden > 1 && l == 1) stage_next(n);
+                    if (hidden > 1 && l == (hidden > 2 ? 2 : 1)) st.ids(n + 3);
                 }
                 if (!ok) break;
             }

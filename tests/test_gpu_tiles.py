@@ -54,3 +54,23 @@ def test_configurations_give_identical_pixels(R, prec, width, hidden):
                         np.testing.assert_array_equal(a, b, err_msg=f"n {n} steps {steps} tuning {tuning}")
     finally:
         A.amnerf_set_tuning(R.ctx, 0, 0, 0)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16", "fp8", "fp8s"])
+@pytest.mark.parametrize("width,hidden", [(32, 1), (64, 1), (32, 2)])
+def test_shallow_networks_over_many_tiles(R, prec, width, hidden):
+    """A hundred tiles and more per worker with one or two hidden layers, where the staging of
+    the next tiles' crossings has the least slack: every wait is met (no timeout in the status
+    word) and a second render gives the same pixels."""
+    cfg = S.CONFIGS["c1"]
+    grid = S.density_grid(S.scene_for(cfg.scene, 1), cfg.G)
+    R.build_tree(grid, cfg.max_depth, cfg.leaf_mass_frac)
+    P = S.xavier_weights(1, S.leaf_mean_density(grid, R.leaf_cells()), width, hidden, cfg.lx, cfg.ld)
+    act = np.full((R.n_leaves, hidden), 2.0, np.float32) if prec == "fp8s" else None
+    R.load_mlps(P, width, hidden, cfg.lx, cfg.ld, "fp8" if act is not None else prec, act_max=act)
+    rays = [torch.from_numpy(np.ascontiguousarray(a)).cuda() for a in S.view_rays(cfg, 1, 0, 800, 700)]
+    first = [t.clone() for t in R.render(*rays, steps=8, cap=64)]
+    R.sync()
+    for a, b in zip(R.render(*rays, steps=8, cap=64), first):
+        assert torch.equal(a, b)
+    R.sync()

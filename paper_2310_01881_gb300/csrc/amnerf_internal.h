@@ -93,7 +93,7 @@ cudaError_t launch_traverse(cudaStream_t s, const float* ro, const float* rd, ui
                             int n_nets, int* err, const uint64_t* mask = nullptr,
                             const uint8_t* fallback = nullptr, float2* root_out = nullptr,
                             const OccArgs& occ = OccArgs(), const HierArgs& hier = HierArgs(),
-                            int depth = kMaxDepth, uint32_t* ray_counter = nullptr);
+                            int depth = kMaxDepth, uint32_t* ray_counter = nullptr, int n_nodes = 0);
 
 // K-b: exclusive scans (crossings and network tiles per leaf) and the grouped scatter.
 // acc (may be NULL) accumulates (crossings, tiles) over the waves of one render.

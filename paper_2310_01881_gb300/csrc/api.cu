@@ -602,7 +602,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
     } else {
         CK(launch_traverse(s, ro, rd, nn, ctx->d_nodes, ctx->d_walk, maxc, ctx->d_nx, ctx->d_xing, ctx->d_xleaf,
                            ctx->d_counts, L, ctx->d_err, mask, fallback, root_out, occ, hier, ctx->tree_depth,
-                           ctx->d_ray_ctr),
+                           ctx->d_ray_ctr, (int)ctx->nodes.size()),
            "traverse launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[1], s);

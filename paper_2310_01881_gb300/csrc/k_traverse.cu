@@ -155,6 +155,7 @@ struct TravArgs {
     int depth;  // stack entries per thread: the tree's depth
     uint32_t* next_ray;  // persistent CTAs: kRayCounters ray counters (see the kernel)
     uint32_t per_warp;   // rays a warp takes at a time: 32, or fewer in a small batch
+    int n_nodes;         // SM: nodes copied to shared memory
 };
 
 // Features compiled into one instantiation of the walk, so that a render keeps in
@@ -354,7 +355,9 @@ __device__ __forceinline__ bool walk_stops(const TravArgs& t, const RayWalk& w, 
 // CTA waits on its slowest ray once, at the end, instead of once per 256 rays (0.415
 // against 0.463 ms at 800x800 x 8).  Six CTAs per SM (40 registers) when the shared
 // memory allows it.
-template <int F>
+// SM: the walk array is read from a copy in shared memory (after the other areas), taken
+// whole at the start.
+template <int F, bool SM>
 __global__ void __launch_bounds__(kTravThreads, 6) k_traverse(const TravArgs t, int n_leaves) {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TravSmem sm;
@@ -368,6 +371,12 @@ __global__ void __launch_bounds__(kTravThreads, 6) k_traverse(const TravArgs t, 
     sm.chk = reinterpret_cast<uint16_t*>(p) + 2 * threadIdx.x;
     if (F & kFVec) p += (size_t)8 * kTravThreads * sizeof(uint16_t);
     sm.nd = reinterpret_cast<uint16_t*>(p) + threadIdx.x;
+    const float2* walk = t.walk;
+    if (SM) {
+        float2* copy = reinterpret_cast<float2*>(p + (size_t)t.depth * kTravThreads * sizeof(uint16_t));
+        for (int i = threadIdx.x; i < t.n_nodes; i += kTravThreads) copy[i] = __ldg(t.walk + i);
+        walk = copy;
+    }
     for (int i = threadIdx.x; i < n_leaves; i += blockDim.x) sm.cnt[i] = 0u;
     __syncthreads();
     const bool pers = t.next_ray != nullptr;
@@ -386,7 +395,7 @@ __global__ void __launch_bounds__(kTravThreads, 6) k_traverse(const TravArgs t, 
         RayWalk w;
         if (r < t.n && walk_init<F>(t, w, r)) {
             while (true) {
-                const float2 sm2 = __ldg(t.walk + w.nd);  // split, meta
+                const float2 sm2 = SM ? walk[w.nd] : __ldg(walk + w.nd);  // split, meta
                 const uint32_t meta = __float_as_uint(sm2.y);
                 const int axis = (int)(meta & 3u) - 1;
                 bool next;
@@ -412,26 +421,37 @@ __global__ void __launch_bounds__(kTravThreads, 6) k_traverse(const TravArgs t, 
 
 // A warp walks until its last ray is done and both sides of every branch its rays take, so a
 // small batch, which leaves the SMs idle, is faster with fewer rays per warp.  Traversal
-// stage with 32 / 16 / 8 / 4 rays per warp: 36.8 / 35.3 / 31.6 / 29.3 us at 9 471 rays,
-// 36.0 / 34.6 / 32.4 / 33.7 at 30 000, 36.4 / 37.7 / 39.1 / 45.9 at 76 800 (256 leaves).
+// stage with 32 / 16 / 8 / 4 rays per warp: 36.4 / 35.0 / 32.2 / 30.0 us at 9 471 rays,
+// 36.7 / 35.3 / 31.9 / 33.2 at 30 000, 36.6 / 37.6 / 39.7 / 46.4 at 76 800 (256 leaves).
+// Its nodes are mostly touched once per SM, so it also walks a copy of the array in shared
+// memory: 27.1 us against 30.0 at 9 471 rays, 44.6 against 48.7 at 10 000 rays and 2 048
+// leaves; larger batches find the nodes in L1 and lose occupancy to the copy (178 against
+// 133 us at 640 000 rays and 2 048 leaves).  The copy stops at 4 095 nodes (32 KB), which
+// leave room for two CTAs per SM.
 uint32_t rays_per_warp(uint32_t n, bool counters) { return !counters || n > 50000u ? 32u : (n > 16000u ? 8u : 4u); }
+constexpr int kWalkCopyNodes = 4095;
 
 using TravKernel = void (*)(const TravArgs, int);
 
 // The sixteen feature combinations, indexed by their flags.
-template <int... Fs>
+template <bool SM, int... Fs>
 struct TravTable {
-    static constexpr TravKernel k[sizeof...(Fs)] = {k_traverse<Fs>...};
+    static constexpr TravKernel k[sizeof...(Fs)] = {k_traverse<Fs, SM>...};
 };
-using Trav16 = TravTable<0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15>;
+using Trav16 = TravTable<false, 0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15>;
+using Trav16S = TravTable<true, 0, 1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15>;
 
 }  // namespace
 
 cudaError_t prepare_traverse() {
     const int smem = (int)trav_smem_bytes(kMaxNets, kMaxDepth, true);
     cudaError_t e = cudaSuccess;
-    for (int f = 0; f < 16 && e == cudaSuccess; ++f)
+    for (int f = 0; f < 16 && e == cudaSuccess; ++f) {
         e = cudaFuncSetAttribute(Trav16::k[f], cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(Trav16S::k[f], cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     smem + (int)(kWalkCopyNodes * sizeof(float2)));
+    }
     return e;
 }
 
@@ -439,16 +459,18 @@ cudaError_t launch_traverse(cudaStream_t s, const float* ro, const float* rd, ui
                             const float2* walk, int maxc, uint8_t* n_x, float2* xing, uint16_t* xleaf,
                             uint32_t* counts, int n_leaves, int* err, const uint64_t* mask, const uint8_t* fallback,
                             float2* root_out, const OccArgs& occ, const HierArgs& hier, int depth,
-                            uint32_t* ray_counter) {
+                            uint32_t* ray_counter, int n_nodes) {
     if (n == 0) return cudaSuccess;
     if (n_leaves < 1 || n_leaves > kMaxNets || depth < 0 || depth > kMaxDepth) return cudaErrorInvalidValue;
     TravArgs t{ro, rd, n, nodes, walk, maxc, n_x, xing, xleaf, counts, err, mask, fallback, root_out, occ, hier,
-               depth > 0 ? depth : 1, ray_counter, rays_per_warp(n, ray_counter != nullptr)};
+               depth > 0 ? depth : 1, ray_counter, rays_per_warp(n, ray_counter != nullptr), n_nodes};
     const int f = ((hier.lod > 0.0f && hier.node_net) ? kFHier : 0) | (mask ? kFMask : 0) |
                   (occ.grid ? kFOcc : 0) | ((maxc & 7) == 0 ? kFVec : 0);
-    const TravKernel kern = Trav16::k[f];
+    const bool sm_walk = t.per_warp < 32 && n_nodes > 0 && n_nodes <= kWalkCopyNodes;
+    const TravKernel kern = sm_walk ? Trav16S::k[f] : Trav16::k[f];
     unsigned blocks = (unsigned)(((uint64_t)n * (32 / t.per_warp) + kTravThreads - 1) / kTravThreads);
-    const size_t smem = trav_smem_bytes(n_leaves, t.depth, (f & kFVec) != 0);
+    const size_t smem = trav_smem_bytes(n_leaves, t.depth, (f & kFVec) != 0) +
+                        (sm_walk ? (size_t)n_nodes * sizeof(float2) : 0);
     if (t.next_ray) {  // persistent: as many CTAs as are resident at once
         int dev = 0, sms = 0, per = 0;
         cudaError_t e = cudaGetDevice(&dev);

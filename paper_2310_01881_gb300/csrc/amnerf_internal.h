@@ -56,6 +56,33 @@ __device__ __forceinline__ float jit_fraction(uint64_t seed, uint64_t key, int k
 }
 #endif
 
+#ifdef __CUDACC__
+// ---- dependent launches ------------------------------------------------------------------
+// A grid launched after another with `pdl` may start once every CTA of that one has called
+// grid_launch (or ended); grid_wait then waits until it has ended and its writes are visible.
+// What such a predecessor wrote is read after grid_wait with loads that go to L2 (__ldcg,
+// cp.async): this grid may have started before it was written.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Such a launch, or an ordinary one.
+template <class... Args>
+inline cudaError_t launch_after(cudaStream_t s, bool pdl, void (*kern)(Args...), unsigned grid, unsigned threads, size_t smem,
+                         Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+#endif
+
 // Error word values written by kernels (first error wins).
 constexpr int kDevErrTimeout = 1;
 constexpr int kDevErrStack = 2;
@@ -93,7 +120,8 @@ cudaError_t launch_traverse(cudaStream_t s, const float* ro, const float* rd, ui
                             int n_nets, int* err, const uint64_t* mask = nullptr,
                             const uint8_t* fallback = nullptr, float2* root_out = nullptr,
                             const OccArgs& occ = OccArgs(), const HierArgs& hier = HierArgs(),
-                            int depth = kMaxDepth, uint32_t* ray_counter = nullptr, int n_nodes = 0);
+                            int depth = kMaxDepth, uint32_t* ray_counter = nullptr, int n_nodes = 0,
+                            bool chain = false);
 
 // K-b: exclusive scans (crossings and network tiles per leaf) and the grouped scatter.
 // acc (may be NULL) accumulates (crossings, tiles) over the waves of one render.
@@ -102,7 +130,11 @@ cudaError_t launch_scan(cudaStream_t s, const uint32_t* counts, int n_leaves, in
 // Both for a whole batch (one launch when it is small).  cursor: zero on entry.
 cudaError_t launch_group(cudaStream_t s, const uint8_t* n_x, const uint16_t* xleaf, uint32_t n_rays, int maxc,
                          const uint32_t* counts, int n_leaves, int cpt, uint32_t* offsets, uint32_t* tile_off,
-                         uint32_t* cursor, uint64_t* stats, uint32_t* order);
+                         uint32_t* cursor, uint64_t* stats, uint32_t* order, bool chain);
+// Whether a batch is grouped in that one launch.  The traversal, the grouping and the network
+// of such a batch are chained: each lets the next start before it has ended (dependent
+// launches), which takes the launch latencies out of a small render.
+bool small_batch(uint32_t n_rays, int maxc);
 // One wave: crossing k of ray r takes part when k_lo <= k < min(n_x[r], k_hi) and
 // alive[r] (alive == NULL: every ray).  count: only the per-leaf totals, added to
 // cursor (zeroed by the caller); else the grouped scatter from the scanned cursor.
@@ -153,6 +185,7 @@ struct MlpArgs {
     float* amax;            // FP32 path, calibration: per leaf x hidden layer, max |input of layer l| (or NULL)
     int act_static;         // E4M3 path: static per-leaf, per-layer activation scales folded into the blob
     uint64_t jitter;        // sample placement: 0 = stratum midpoints, else the stratified jitter's seed
+    bool chain;             // dependent launch after the grouping (tensor-core kernels)
 };
 cudaError_t launch_mlp_simt(cudaStream_t s, const MlpArgs& a, int grid);
 cudaError_t launch_mlp_tc(cudaStream_t s, const MlpArgs& a, int grid, int prec);

@@ -562,6 +562,9 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
     HierArgs hier;
     hier.lod = p->lod;
     hier.node_net = ctx->d_node_net;
+    // a small batch's launches are chained; not with other work between them
+    const bool chain = small_batch(nn, maxc) && !cin && !ctx->timing && !(p->ert_wave > 0) && !bins_out &&
+                       ctx->tuning.schedule != AMNERF_SCHED_PER_LEAF;
     if (ctx->timing) cudaEventRecord(ctx->ev[0], s);
     // ray counters, statistics, the L counts and the L cursors lie together: one memset
     ctx->d_cursor = ctx->d_counts + L;
@@ -602,7 +605,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
     } else {
         CK(launch_traverse(s, ro, rd, nn, ctx->d_nodes, ctx->d_walk, maxc, ctx->d_nx, ctx->d_xing, ctx->d_xleaf,
                            ctx->d_counts, L, ctx->d_err, mask, fallback, root_out, occ, hier, ctx->tree_depth,
-                           ctx->d_ray_ctr, (int)ctx->nodes.size()),
+                           ctx->d_ray_ctr, (int)ctx->nodes.size(), chain),
            "traverse launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[1], s);
@@ -618,7 +621,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         if (st != AMNERF_OK) return st;
     } else {
         CK(launch_group(s, ctx->d_nx, ctx->d_xleaf, nn, maxc, ctx->d_counts, L, kTileRows / steps, ctx->d_offsets,
-                        ctx->d_tile_off, ctx->d_cursor, ctx->d_stats, ctx->d_order),
+                        ctx->d_tile_off, ctx->d_cursor, ctx->d_stats, ctx->d_order, chain),
            "grouping launch");
     }
     if (ctx->timing) cudaEventRecord(ctx->ev[2], s);
@@ -652,6 +655,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         a.amax = ctx->calibrating ? ctx->d_amax : nullptr;
         a.act_static = ctx->act_static ? 1 : 0;
         a.jitter = p->jitter_seed;
+        a.chain = chain;
         a.tile_counter = reinterpret_cast<uint32_t*>(ctx->d_stats + 6);
         a.t_begin = 0;
         a.t_end = 0xffffffffu;

@@ -200,12 +200,14 @@ __global__ void __launch_bounds__(kRayScatterThreads) k_scatter_rays(const uint8
     uint32_t* s_cnt = sm;
     uint32_t* s_base = sm + n_leaves;
     if (SCAN) {
+        grid_launch();
+        grid_wait();
         __shared__ uint32_t s_w[2][kRayScatterThreads / 32];
         const int per = (n_leaves + kRayScatterThreads - 1) / kRayScatterThreads;
         const int i0 = min((int)threadIdx.x * per, n_leaves), i1 = min(i0 + per, n_leaves);
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
         // the counts as coalesced loads, then each thread its run of them
-        for (int i = threadIdx.x; i < n_leaves; i += kRayScatterThreads) s_base[i] = __ldg(sc.counts + i);
+        for (int i = threadIdx.x; i < n_leaves; i += kRayScatterThreads) s_base[i] = __ldcg(sc.counts + i);
         __syncthreads();
         uint32_t c = 0, t = 0;
         for (int i = i0; i < i1; ++i) {
@@ -251,11 +253,11 @@ __global__ void __launch_bounds__(kRayScatterThreads) k_scatter_rays(const uint8
     for (int i = threadIdx.x; i < n_leaves; i += blockDim.x) s_cnt[i] = 0u;
     __syncthreads();
     const uint32_t r = blockIdx.x * (uint32_t)kRayScatterThreads + threadIdx.x;
-    const int nx = r < n_rays ? min((int)__ldg(n_x + r), maxc) : 0;
+    const int nx = r < n_rays ? min((int)__ldcg(n_x + r), maxc) : 0;
     const size_t base = (size_t)r * (size_t)maxc;
     if (VEC) {
         for (int k0 = 0; k0 < nx; k0 += 8) {
-            const uint4 v = __ldg(reinterpret_cast<const uint4*>(xleaf + base + k0));
+            const uint4 v = __ldcg(reinterpret_cast<const uint4*>(xleaf + base + k0));
             const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -269,7 +271,7 @@ __global__ void __launch_bounds__(kRayScatterThreads) k_scatter_rays(const uint8
         }
     } else {
         for (int k = 0; k < nx; ++k) {
-            const uint32_t id = __ldg(xleaf + base + k);
+            const uint32_t id = __ldcg(xleaf + base + k);
             s_id[k * kRayScatterThreads] = (uint16_t)id;
             s_rk[k * kRayScatterThreads] = (uint16_t)warp_rank(s_cnt, id);
         }
@@ -348,12 +350,16 @@ cudaError_t launch_scan(cudaStream_t s, const uint32_t* counts, int n_leaves, in
 // beyond, the scans repeated by thousands of CTAs would cost more than the launch saved.
 constexpr unsigned kScanInScatter = 300;
 
+bool small_batch(uint32_t n_rays, int maxc) {
+    return n_rays > 0 && maxc <= kRayScatterMaxc && n_rays <= kScanInScatter * kRayScatterThreads;
+}
+
 cudaError_t launch_group(cudaStream_t s, const uint8_t* n_x, const uint16_t* xleaf, uint32_t n_rays, int maxc,
                          const uint32_t* counts, int n_leaves, int cpt, uint32_t* offsets, uint32_t* tile_off,
-                         uint32_t* cursor, uint64_t* stats, uint32_t* order) {
+                         uint32_t* cursor, uint64_t* stats, uint32_t* order, bool chain) {
     const uint64_t n_slots = (uint64_t)n_rays * (uint64_t)maxc;
     const unsigned blocks = (n_rays + kRayScatterThreads - 1) / kRayScatterThreads;
-    const bool fused = n_slots > 0 && maxc <= kRayScatterMaxc && blocks <= kScanInScatter;
+    const bool fused = n_slots > 0 && small_batch(n_rays, maxc);
     if (!fused) {
         const cudaError_t e = launch_scan(s, counts, n_leaves, cpt, offsets, tile_off, cursor, stats);
         if (e != cudaSuccess || n_slots == 0) return e;
@@ -363,10 +369,11 @@ cudaError_t launch_group(cudaStream_t s, const uint8_t* n_x, const uint16_t* xle
                             2 * sizeof(uint16_t) * (size_t)maxc * kRayScatterThreads;
         const ScanArgs sc{counts, cpt, offsets, tile_off, stats};
         const bool vec = (maxc & 7) == 0;
-        auto* kern = fused ? (vec ? k_scatter_rays<true, true> : k_scatter_rays<false, true>)
+        void (*kern)(const uint8_t*, const uint16_t*, uint32_t, int, uint32_t*, uint32_t*, int, const ScanArgs) =
+            fused ? (vec ? k_scatter_rays<true, true> : k_scatter_rays<false, true>)
                            : (vec ? k_scatter_rays<true, false> : k_scatter_rays<false, false>);
-        kern<<<blocks, kRayScatterThreads, smem, s>>>(n_x, xleaf, n_rays, maxc, cursor, order, n_leaves, sc);
-        return cudaGetLastError();
+        return launch_after(s, fused && chain, kern, blocks, (unsigned)kRayScatterThreads, smem, n_x, xleaf, n_rays,
+                            maxc, cursor, order, n_leaves, sc);
     }
     const uint64_t per = (uint64_t)kScatterThreads * kScatterItems;
     const unsigned sblocks = (unsigned)((n_slots + per - 1) / per);

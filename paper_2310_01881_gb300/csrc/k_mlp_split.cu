@@ -216,6 +216,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
+    grid_wait();  // a chained launch: the crossings and their grouping
 
     const bool aux = warp >= 4 * kGroups * kTPR;
     const int gi = aux ? q : warp >> 3;  // this warp's group (aux: warp i of the last warpgroup serves group i)
@@ -236,7 +237,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
         return ok;
     };
     // this CTA's contiguous range of tiles; group i takes tiles t0 + i, t0 + i + kGroups, ...
-    const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
+    const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)__ldcg(g.stats + 1) : g.t_end;
     const uint32_t span = t_end > g.t_begin ? t_end - g.t_begin : 0u;
     const uint32_t per = (span + gridDim.x - 1) / gridDim.x;
     const uint32_t t0 = min(g.t_begin + blockIdx.x * per, t_end);
@@ -271,7 +272,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
                 }
                 if (!wait(bar_w, ph_w)) break;
                 ph_w ^= 1u;
-                const uint32_t seg_end = min(t1, __ldg(g.tile_off + leaf + 1));
+                const uint32_t seg_end = min(t1, __ldcg(g.tile_off + leaf + 1));
                 // this group's tiles below seg_end: numbers n with t0 + gi + kGroups n < seg_end
                 for (; t0 + (uint32_t)gi + kGroups * n < seg_end && ok; ++n) {
                     // layer 0: per chunk the small products, after the last chunk the large ones
@@ -561,14 +562,9 @@ cudaError_t prepare_w(int max_smem) {
 template <int W>
 cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid, size_t smem) {
     const bool hc = a.hidden == kHiddenFor<W>;
-    if (a.jitter) {
-        if (hc) k_mlp_split<W, kHiddenFor<W>, true><<<grid, kThreads, smem, s>>>(a);
-        else k_mlp_split<W, 0, true><<<grid, kThreads, smem, s>>>(a);
-    } else {
-        if (hc) k_mlp_split<W, kHiddenFor<W>, false><<<grid, kThreads, smem, s>>>(a);
-        else k_mlp_split<W, 0, false><<<grid, kThreads, smem, s>>>(a);
-    }
-    return cudaGetLastError();
+    void (*kern)(MlpArgs) = a.jitter ? (hc ? k_mlp_split<W, kHiddenFor<W>, true> : k_mlp_split<W, 0, true>)
+                                     : (hc ? k_mlp_split<W, kHiddenFor<W>, false> : k_mlp_split<W, 0, false>);
+    return launch_after(s, a.chain, kern, (unsigned)grid, (unsigned)kThreads, smem, a);
 }
 
 }  // namespace

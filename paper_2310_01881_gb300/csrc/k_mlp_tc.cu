@@ -281,6 +281,7 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = sh->tmem_base;
+    grid_wait();  // a chained launch: the crossings and their grouping
 
     // Warpgroups 0 .. n_groups - 1 compute; warp i of the last one serves group i: it stages
     // the crossings, loads the weights and issues the MMAs, so that nothing of that sits in
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
             const uint64_t desc_wo = sdesc(w_addr + (uint32_t)lay.wo, (uint32_t)lay.khead * 16u);
             const uint64_t desc_bb = sdesc(w_addr + (uint32_t)lay.bb, (uint32_t)kBiasK * 16u);
             const uint8_t* wall = reinterpret_cast<const uint8_t*>(g.weights);
-            const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)g.stats[1] : g.t_end;
+            const uint32_t t_end = g.t_end == 0xffffffffu ? (uint32_t)__ldcg(g.stats + 1) : g.t_end;
             uint32_t t_stop = t_end, t_step = 1, t_next;
             {
                 const uint32_t workers = gridDim.x * (uint32_t)n_groups;
@@ -1299,7 +1300,9 @@ cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid) {
     if (smem < (size_t)max_smem / 2 + 1024) smem = (size_t)max_smem / 2 + 1024;
     const bool hc = a.hidden == kHiddenFor<W>;
     const bool st = F8 && a.act_static;
-#define AMNERF_TC(ST_, HC_, J_) k_mlp_tc<W, F8, ST_, HC_, J_><<<grid, 128 * (groups + 1), smem, s>>>(a, groups, cols)
+    cudaError_t e = cudaSuccess;
+#define AMNERF_TC(ST_, HC_, J_)                                                                                  \
+    e = launch_after(s, a.chain, k_mlp_tc<W, F8, ST_, HC_, J_>, (unsigned)grid, 128u * (groups + 1), smem, a, groups, cols)
     if (a.jitter) {
         if (st) { if (hc) AMNERF_TC(F8, kHiddenFor<W>, true); else AMNERF_TC(F8, 0, true); }
         else { if (hc) AMNERF_TC(false, kHiddenFor<W>, true); else AMNERF_TC(false, 0, true); }
@@ -1308,7 +1311,7 @@ cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid) {
         else { if (hc) AMNERF_TC(false, kHiddenFor<W>, false); else AMNERF_TC(false, 0, false); }
     }
 #undef AMNERF_TC
-    return cudaGetLastError();
+    return e;
 }
 
 }  // namespace

@@ -621,11 +621,6 @@ struct GradSmem {
     float loss[kGThreads / 32];
 };
 
-// What an earlier step wrote is read after grid_wait with loads that go to L2 (__ldcg): this
-// grid may have started before it was written.
-__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // acc[i] += w * v[i] over the four rays of v.
 __device__ __forceinline__ void fma4(float w, const float4& v, float (&acc)[4]) {
     acc[0] = fmaf(w, v.x, acc[0]);
@@ -876,24 +871,6 @@ __global__ void __launch_bounds__(256) k_prop_reduce(const float* __restrict__ p
 }
 constexpr int kReduceBlocks = (NPAR + 1 + 31) / 32;
 static_assert(kReduceBlocks * 32 <= kPartStride, "the last block stays inside a partial");
-
-// A launch that may start before its predecessor in the stream has ended (pdl; the kernel
-// then waits for it itself), or an ordinary one.
-template <class... Args>
-cudaError_t launch_after(cudaStream_t s, bool pdl, void (*kern)(Args...), unsigned grid, unsigned threads, size_t smem,
-                         Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
 
 }  // namespace
 

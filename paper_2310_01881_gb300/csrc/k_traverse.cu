@@ -156,6 +156,7 @@ struct TravArgs {
     uint32_t* next_ray;  // persistent CTAs: kRayCounters ray counters (see the kernel)
     uint32_t per_warp;   // rays a warp takes at a time: 32, or fewer in a small batch
     int n_nodes;         // SM: nodes copied to shared memory
+    bool chain;          // the grouping may start before the traversal has ended
 };
 
 // Features compiled into one instantiation of the walk, so that a render keeps in
@@ -360,6 +361,7 @@ __device__ __forceinline__ bool walk_stops(const TravArgs& t, const RayWalk& w, 
 template <int F, bool SM>
 __global__ void __launch_bounds__(kTravThreads, 6) k_traverse(const TravArgs t, int n_leaves) {
     extern __shared__ __align__(16) unsigned char s_raw[];
+    if (t.chain) grid_launch();
     TravSmem sm;
     unsigned char* p = s_raw;
     sm.cnt = reinterpret_cast<uint32_t*>(p);
@@ -459,11 +461,11 @@ cudaError_t launch_traverse(cudaStream_t s, const float* ro, const float* rd, ui
                             const float2* walk, int maxc, uint8_t* n_x, float2* xing, uint16_t* xleaf,
                             uint32_t* counts, int n_leaves, int* err, const uint64_t* mask, const uint8_t* fallback,
                             float2* root_out, const OccArgs& occ, const HierArgs& hier, int depth,
-                            uint32_t* ray_counter, int n_nodes) {
+                            uint32_t* ray_counter, int n_nodes, bool chain) {
     if (n == 0) return cudaSuccess;
     if (n_leaves < 1 || n_leaves > kMaxNets || depth < 0 || depth > kMaxDepth) return cudaErrorInvalidValue;
     TravArgs t{ro, rd, n, nodes, walk, maxc, n_x, xing, xleaf, counts, err, mask, fallback, root_out, occ, hier,
-               depth > 0 ? depth : 1, ray_counter, rays_per_warp(n, ray_counter != nullptr), n_nodes};
+               depth > 0 ? depth : 1, ray_counter, rays_per_warp(n, ray_counter != nullptr), n_nodes, chain};
     const int f = ((hier.lod > 0.0f && hier.node_net) ? kFHier : 0) | (mask ? kFMask : 0) |
                   (occ.grid ? kFOcc : 0) | ((maxc & 7) == 0 ? kFVec : 0);
     const bool sm_walk = t.per_warp < 32 && n_nodes > 0 && n_nodes <= kWalkCopyNodes;

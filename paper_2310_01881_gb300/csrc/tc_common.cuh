@@ -384,7 +384,7 @@ __device__ __forceinline__ int leaf_of_tile_warp(const uint32_t* __restrict__ ti
     while (hi - lo > 1) {  // tile_off[lo] <= t < tile_off[hi]
         const int step = (hi - lo + 31) >> 5;
         const int i = lo + step * lane;
-        const bool le = i < hi && __ldg(tile_off + i) <= t;  // lane 0: true
+        const bool le = i < hi && __ldcg(tile_off + i) <= t;  // lane 0: true
         const int k = __popc(__ballot_sync(0xffffffffu, le)) - 1;
         lo += step * k;
         hi = min(hi, lo + step);
@@ -447,10 +447,10 @@ struct Stager {
         if (any) {
             if (t_next >= lk_t1) {
                 lk_leaf = leaf_of_tile_warp(g.tile_off, lk_leaf + 1, g.n_leaves, t_next);
-                lk_t0 = __ldg(g.tile_off + lk_leaf);
-                lk_t1 = __ldg(g.tile_off + lk_leaf + 1);
-                lk_x0 = __ldg(g.offsets + lk_leaf);
-                lk_x1 = __ldg(g.offsets + lk_leaf + 1);
+                lk_t0 = __ldcg(g.tile_off + lk_leaf);
+                lk_t1 = __ldcg(g.tile_off + lk_leaf + 1);
+                lk_x0 = __ldcg(g.offsets + lk_leaf);
+                lk_x1 = __ldcg(g.offsets + lk_leaf + 1);
             }
             for (int c = lane; c < cpt; c += 32) {
                 const uint32_t at = lk_x0 + (t_next - lk_t0) * (uint32_t)cpt + (uint32_t)c;

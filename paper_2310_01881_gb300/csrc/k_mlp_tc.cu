@@ -37,13 +37,13 @@
 // next tile's layer-0 accumulator and activated and stored under that tile's layer 2.
 //
 // A tile's chain is shortened from both ends (4 x 64 BF16 network, 8 views of 800 x 800:
-// network step 12.3 -> 9.5 ms; E4M3 with static scales 12.2 -> 8.6 ms):
+// network step 12.3 -> 9.3 ms; E4M3 with static scales 12.2 -> 8.6 ms):
 //   - what does not need a row's thread sits in one auxiliary warp per group (the fifth
 //     warpgroup): it stages crossing ids, intervals and rays in shared memory tiles ahead
 //     (cp.async), loads the weights and issues the MMAs.  Staging alone gave 12.3 -> 11.0:
 //     the two dependent loads had cost each tile one to two DRAM latencies, as a load into
 //     registers is waited for before the block that issues it is left.  The issue from
-//     warps of its own, and mbarriers in place of group barriers, gave 11.0 -> 9.5.
+//     warps of its own, and mbarriers in place of group barriers, gave 11.0 -> 9.3 (tensor pipe 46 -> 61 % busy, issue 53 -> 65 %).
 //   - the compute warps encode tile t + 1 while tile t's layers run, and store its input
 //     into TMEM columns that are free by then (see kGroupCols).
 //

@@ -119,18 +119,34 @@ __device__ __forceinline__ float2 bf16x2_floats(uint32_t p) {
     return make_float2(__uint_as_float(p << 16), __uint_as_float(p & 0xffff0000u));
 }
 
-// (v0, v1) = h + m + l, two BF16 per word.
+// Two BF16 per word, to nearest, a value beyond the largest finite BF16 to that one.
+__device__ __forceinline__ uint32_t pack_bf16_sat(float lo, float hi) {
+    uint32_t d;
+    asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(d) : "f"(hi), "f"(lo));
+    return d;
+}
+
+// (v0, v1) = h + m + l, two BF16 per word.  h and m saturate: a value above the largest BF16
+// stays exact (h + m), and an infinite activation becomes three times that value, whose
+// products keep its sign and overflow again -- inf - inf would make m NaN and, with it, pixels
+// that FP32 arithmetic gives as opaque.
 __device__ __forceinline__ void split3(float v0, float v1, uint32_t& h, uint32_t& m, uint32_t& l) {
     const float2 neg = make_float2(-1.0f, -1.0f);
-    h = pack_bf16(v0, v1);
+    h = pack_bf16_sat(v0, v1);
     const float2 r = fma2v(bf16x2_floats(h), neg, make_float2(v0, v1));
-    m = pack_bf16(r.x, r.y);
+    m = pack_bf16_sat(r.x, r.y);
     const float2 s = fma2v(bf16x2_floats(m), neg, r);
-    l = pack_bf16(s.x, s.y);
+    l = pack_bf16_sat(s.x, s.y);
 }
 
 __device__ __forceinline__ float softplus_f32(float z) { return z > 20.0f ? z : log1pf(expf(z)); }
 __device__ __forceinline__ float sigmoid_f32(float z) { return 1.0f / (1.0f + expf(-z)); }
+
+// BF16 to nearest; a finite value that would round to infinity becomes the largest BF16.
+__device__ __forceinline__ __nv_bfloat16 bf16_sat(float v) {
+    constexpr float kMax = 3.38953139e38f;  // 0x7f7f0000
+    return __float2bfloat16_rn(fminf(fmaxf(v, -kMax), kMax));
+}
 
 // The FP32 SIMT blob (transposed matrices, see k_mlp_simt.cu) of every network as split
 // operands, one element per thread and step; networks over blockIdx.y.
@@ -163,7 +179,7 @@ __global__ void k_split_pack(const float* __restrict__ simt, size_t simt_stride,
             const int e = i - n0 - nh - no, l = e / (W * kBiasK), n = (e / kBiasK) % W, k = e % kBiasK;
             const int p = k - (kOnesCol - kOnesStep);  // which part this K column carries
             const float b = src[(size_t)(kIn + 1) * W + (size_t)l * (W * W + W) + (size_t)W * W + n];
-            const float h = __bfloat162float(__float2bfloat16_rn(b)), m = __bfloat162float(__float2bfloat16_rn(b - h));
+            const float h = __bfloat162float(bf16_sat(b)), m = __bfloat162float(__float2bfloat16_rn(b - h));
             v = p == 0 ? h : (p == 1 ? m : (p == 2 ? b - h - m : 0.0f));
             *reinterpret_cast<__nv_bfloat16*>(dst + lay.bb + (size_t)l * W * kBiasK * 2 + cm_offset(n, k, kBiasK)) =
                 __float2bfloat16_rn(v);
@@ -174,7 +190,7 @@ __global__ void k_split_pack(const float* __restrict__ simt, size_t simt_stride,
                 src[(size_t)(kIn + 1) * W + (size_t)(hidden - 1) * (W * W + W) + 4 * W + n];
             continue;
         }
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const __nv_bfloat16 h = bf16_sat(v);
         const float r = v - __bfloat162float(h);
         const __nv_bfloat16 m = __float2bfloat16_rn(r);
         *reinterpret_cast<__nv_bfloat16*>(dst + at) = h;

@@ -88,3 +88,27 @@ def test_split_network_outputs_against_64_bits(R):
     err = np.abs(got - want) / np.maximum(np.abs(want), 1.0)
     print(f"network outputs: max error {err.max():.2e}, rms {np.sqrt((err ** 2).mean()):.2e}")
     assert err.max() < 1e-4
+
+
+@pytest.mark.parametrize("width,hidden", [(32, 1), (32, 2), (64, 4)])
+def test_split_networks_overflow_as_fp32_does(R, width, hidden):
+    """Weights beyond the largest BF16 and activations that overflow FP32: an infinite density is
+    opaque and infinite logits saturate, as in the oracle (no NaN from the split)."""
+    cfg = dataclasses.replace(S.CONFIGS["c1"], width=width, hidden=hidden)
+    grid = S.density_grid(S.scene_for(cfg.scene, 2), cfg.G)
+    tree = O.build_tree(grid, cfg.max_depth, cfg.leaf_mass_frac)
+    R.build_tree(grid, cfg.max_depth, cfg.leaf_mass_frac)
+    parts = [np.zeros(width * 90), np.full(width, 3.4e38)]
+    for _ in range(hidden - 1):
+        parts += [np.full(width * width, 0.5), np.zeros(width)]
+    parts += [np.repeat([0.1, 0.1, -0.1, -0.2], width), np.zeros(4)]
+    P = np.tile(np.concatenate(parts).astype(np.float32), (tree.n_leaves, 1))
+    R.load_mlps(P, width, hidden, cfg.lx, cfg.ld, "fp32")
+    o, d = S.view_rays(cfg, 2, 0)
+    o, d = o[1500:2200], d[1500:2200]
+    got = [t.cpu().numpy() for t in R.render(torch.from_numpy(o).cuda(), torch.from_numpy(d).cuda(), steps=8, cap=64)]
+    R.sync()
+    ref = O.render(tree, P, width, hidden, cfg.lx, cfg.ld, o, d, 8, 64, mode=1, threads=8)
+    assert ref["opacity"].max() == 1.0 and np.isfinite(ref["rgb"]).all()
+    for name, a in zip(("rgb", "depth", "opacity"), got):
+        assert np.abs(a - ref[name]).max() <= 1e-5, name

@@ -57,7 +57,7 @@ typedef enum {
 } amnerf_status;
 
 typedef enum {
-    AMNERF_FP32 = 0,     /* plain path: FP32 SIMT network */
+    AMNERF_FP32 = 0,     /* plain path: FP32 network (tensor cores on exactly split operands, or FP32 SIMT) */
     AMNERF_BF16 = 1,     /* tcgen05 tensor cores, BF16 operands, FP32 accumulation */
     AMNERF_FP8E4M3 = 2   /* tcgen05, E4M3 operands with per-channel scales, FP32 accumulation */
 } amnerf_precision;

@@ -1,4 +1,5 @@
-// k_mlp_simt.cu -- K-c, plain FP32 path: per-leaf networks on CUDA cores.
+// k_mlp_simt.cu -- K-c, FP32 networks on CUDA cores: calibration, and the shapes that
+// k_mlp_split.cu does not take (there the tensor cores are 5.8x faster at the same error).
 //
 // Network (Sec. 3.1 F_Theta, one small same-shaped MLP per leaf, Sec. 3.2 and 4.1):
 // input gamma_lx(x) ++ gamma_ld(d) with gamma_L(p) = [p, sin(pi 2^k p), cos(pi 2^k p)]

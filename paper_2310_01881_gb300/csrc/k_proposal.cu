@@ -225,8 +225,8 @@ __device__ __forceinline__ void tile_layer(const float (*in)[kRays], const float
 // true).  The 64 depth masses are sorted (sorting network, descending) and walked
 // in that order, so the running sum sees the same values in the same order as a
 // repeated arg-max; the background enters before the first depth mass it strictly
-// exceeds.  The walk ends at the last kept mass tau, of which the first c_tau bins
-// (lowest indices) with q == tau are kept along with every bin with q > tau.
+// exceeds.  The walk ends at the last kept mass tau; every bin with q > tau is kept and as
+// many of those with q == tau (lowest indices first) as make up the number taken.
 __device__ __forceinline__ bool select_bins(const float (*QB)[kRays], const float (*QA)[kRays], int t,
                                             float coverage, int max_bins, uint64_t& mk) {
 #define Q_(b) ((b) < 32 ? QB[(b)][t] : QA[(b)][t])
@@ -253,34 +253,35 @@ __device__ __forceinline__ bool select_bins(const float (*QB)[kRays], const floa
         }
     }
     const float vbg = Q_(64);
-    bool bg_taken = false, fb = false;
+    // The walk, without branches inside a block of 8 masses: the background is added in
+    // front of the first mass it exceeds, a mass is taken while the sum is below the
+    // coverage (a sum that has reached it stays there, so nothing after it is taken), and
+    // more than max_bins taken is the fallback.  Three compares and branches per mass had made
+    // the walk cost as much as the sort: 33.2 M rays at coverage 0.99 and 64 bins took 5.4 ms,
+    // 3.2 with this form (16 bins at most: 3.3 and 2.9).
     float cum = 0.0f, tau = 0.0f;
-    int kept = 0, c_tau = 0;
+    int kept = 0;
+    bool above = false;  // vbg > the mass before
 #pragma unroll
-    for (int p = 0; p < 64; ++p) {
-        if (!bg_taken && vbg > v[p]) {
-            if (!(cum < coverage)) break;
-            cum += vbg;
-            bg_taken = true;
+    for (int p0 = 0; p0 < 64; p0 += 8) {
+        if (p0 > max_bins || !(cum < coverage)) break;
+#pragma unroll
+        for (int p = p0; p < p0 + 8; ++p) {
+            const bool now = vbg > v[p];
+            if (now && !above) cum += vbg;
+            above = now;
+            if (cum < coverage) {
+                cum += v[p];
+                tau = v[p];
+                ++kept;
+            }
         }
-        if (!(cum < coverage)) break;
-        cum += v[p];
-        if (kept == max_bins) {
-            fb = true;
-            break;
-        }
-        if (kept > 0 && v[p] == tau) {
-            ++c_tau;
-        } else {
-            tau = v[p];
-            c_tau = 1;
-        }
-        ++kept;
     }
     mk = 0;
-    if (fb || kept == 0) return fb;
+    if (kept > max_bins) return true;
+    if (kept == 0) return false;
     // Without a tie cut off by the walk the kept bins are those with q >= tau (their number
-    // says so); otherwise the first c_tau of the ties.  The first form is a compare and a
+    // says so); otherwise the first of the ties.  The first form is a compare and a
     // select per bin with no chain through the tie count, in a loop short enough to leave the
     // registers to the sort: a 1920 x 1080 proposal render (x1000 densities, coverage 0.95)
     // took 1 033 us with the second form alone, 922 with both.
@@ -294,14 +295,26 @@ __device__ __forceinline__ bool select_bins(const float (*QB)[kRays], const floa
         mk = (uint64_t)lo | ((uint64_t)hi << 32);
         return false;
     }
-    int eq = 0;
-#pragma unroll
-    for (int b = 0; b < 64; ++b) {
-        const float q = Q_(b);
-        const bool take = q > tau || (q == tau && eq < c_tau);
-        eq += (q == tau && take) ? 1 : 0;
-        mk |= take ? (1ull << b) : 0ull;
+    int ties = kept;  // the first `ties` bins with q == tau are kept
+#pragma unroll 4
+    for (int b = 0; b < 32; ++b) ties -= (QB[b][t] > tau ? 1 : 0) + (QA[b + 32][t] > tau ? 1 : 0);
+    lo = 0u;
+    hi = 0u;
+#pragma unroll 4
+    for (int b = 0; b < 32; ++b) {
+        const float q = QB[b][t];
+        const bool take = q > tau || (q == tau && ties > 0);
+        ties -= q == tau ? 1 : 0;
+        lo |= take ? 1u << b : 0u;
     }
+#pragma unroll 4
+    for (int b = 0; b < 32; ++b) {
+        const float q = QA[b + 32][t];
+        const bool take = q > tau || (q == tau && ties > 0);
+        ties -= q == tau ? 1 : 0;
+        hi |= take ? 1u << b : 0u;
+    }
+    mk = (uint64_t)lo | ((uint64_t)hi << 32);
     return false;
 #undef Q_
 }

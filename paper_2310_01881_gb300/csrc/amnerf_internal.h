@@ -175,7 +175,8 @@ struct MlpArgs {
     const float* ro;
     const float* rd;
     const void* weights;    // packed per leaf, layout depends on precision
-    size_t leaf_stride;     // bytes per leaf
+    const float* weights_fp32;  // FP32 networks: the SIMT kernel's blob (the split kernel's `weights` is another)
+    size_t leaf_stride;     // bytes per leaf (FP32: of weights_fp32)
     int width, hidden, lx, ld, k0;
     int steps, maxc, cap;
     uint32_t maxc_magic;    // ceil(2^32 / maxc) (maxc >= 2): id / maxc by multiply-high (see div_maxc)

@@ -638,6 +638,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         a.ro = ro;
         a.rd = rd;
         a.weights = ctx->d_weights;
+        a.weights_fp32 = static_cast<const float*>(ctx->d_weights);
         a.leaf_stride = ctx->leaf_stride;
         a.width = ctx->desc.width;
         a.hidden = ctx->desc.hidden;

@@ -126,17 +126,23 @@ __device__ __forceinline__ uint32_t pack_bf16_sat(float lo, float hi) {
     return d;
 }
 
-// (v0, v1) = h + m + l, two BF16 per word.  h and m saturate: a value above the largest BF16
-// stays exact (h + m), and an infinite activation becomes three times that value, whose
-// products keep its sign and overflow again -- inf - inf would make m NaN and, with it, pixels
-// that FP32 arithmetic gives as opaque.
+// (v0, v1) = h + m + l, two BF16 per word.  h saturates, so that a value above the largest BF16
+// stays exact (h + m).  Of an infinity or a NaN at least one part is NaN (m or l of inf - inf),
+// so all that a sample's network computes from it is NaN: see fp32_sample.
 __device__ __forceinline__ void split3(float v0, float v1, uint32_t& h, uint32_t& m, uint32_t& l) {
     const float2 neg = make_float2(-1.0f, -1.0f);
     h = pack_bf16_sat(v0, v1);
     const float2 r = fma2v(bf16x2_floats(h), neg, make_float2(v0, v1));
-    m = pack_bf16_sat(r.x, r.y);
+    m = pack_bf16(r.x, r.y);
     const float2 s = fma2v(bf16x2_floats(m), neg, r);
-    l = pack_bf16_sat(s.x, s.y);
+    l = pack_bf16(s.x, s.y);
+}
+
+// max(v, 0), or NaN.
+__device__ __forceinline__ float relu_nan(float v) {
+    float r;
+    asm("max.NaN.f32 %0, %1, 0f00000000;" : "=f"(r) : "f"(v));
+    return r;
 }
 
 __device__ __forceinline__ float softplus_f32(float z) { return z > 20.0f ? z : log1pf(expf(z)); }
@@ -199,9 +205,83 @@ __global__ void k_split_pack(const float* __restrict__ simt, size_t simt_stride,
     }
 }
 
+// Sample j of crossing id by a whole converged warp in FP32, from k_mlp_simt's copy of the leaf's
+// weights and with its operations in its order: each lane holds W / 32 activations, a layer's
+// inputs go round by shuffles.  For samples whose tensor-core result is NaN: an activation
+// overflowed (or the input is not finite), and the split of an infinity has no products that add
+// up to FP32's.  Microseconds per sample; out of line, so that it costs the kernel no registers.
+template <int W, bool JIT>
+__device__ __noinline__ void fp32_sample(const MlpArgs& g, int leaf, int hidden, uint32_t id, int j) {
+    constexpr int R = W / 32;
+    const int lane = threadIdx.x & 31;
+    const float* w = g.weights_fp32 + (size_t)leaf * (g.leaf_stride / sizeof(float));
+    const uint32_t ray = id / (uint32_t)g.maxc;
+    const float2 xi = __ldcg(g.xing + id);
+    float x[3], d[3], o[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        o[a] = __ldg(g.ro + 3 * (size_t)ray + a);
+        d[a] = __ldg(g.rd + 3 * (size_t)ray + a);
+    }
+    const float delta = __fmul_rn(__fsub_rn(xi.y, xi.x), __frcp_rn((float)g.steps));
+    float u = 0.5f;
+    if (JIT)
+        u = jit_fraction(g.jitter, jit_ray_key(g.jitter, o, d), (int)(id - ray * (uint32_t)g.maxc), g.steps, j);
+    const float tj = __fadd_rn(xi.x, __fmul_rn(__fadd_rn((float)j, u), delta));
+#pragma unroll
+    for (int a = 0; a < 3; ++a) x[a] = __fadd_rn(o[a], __fmul_rn(tj, d[a]));
+    float in[3];  // inputs lane, lane + 32, lane + 64
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        const int f = lane + 32 * i, e = f < 63 ? f - 3 : f - 66;  // e < 0: the coordinate itself
+        const int a = f < 3 ? f : (f >= 63 && f < 66 ? f - 63 : e % 3);
+        const float p = f < 63 ? (a == 0 ? x[0] : (a == 1 ? x[1] : x[2])) : (a == 0 ? d[0] : (a == 1 ? d[1] : d[2]));
+        in[i] = p;
+        if (e >= 0 && f < kIn) {
+            float sn, cs;
+            sincospif(p * (float)(1 << (e / 6)), &sn, &cs);
+            in[i] = e % 6 < 3 ? sn : cs;
+        }
+    }
+    float h[R];
+    auto layer = [&](const float* v, int kin) {
+        const float* b = w + (size_t)kin * W;
+        float acc[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = __ldg(b + lane + 32 * r);
+        for (int k0 = 0; k0 < kin; k0 += 32) {
+            const float vk = k0 == 0 ? v[0] : (k0 == 32 ? v[1] : v[2]);
+#pragma unroll 8
+            for (int k = 0; k < min(32, kin - k0); ++k) {
+                const float a = __shfl_sync(0xffffffffu, vk, k);
+#pragma unroll
+                for (int r = 0; r < R; ++r) acc[r] = fmaf(a, __ldg(w + (size_t)(k0 + k) * W + lane + 32 * r), acc[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) h[r] = fmaxf(acc[r], 0.0f);
+        w = b + W;
+    };
+    layer(in, kIn);
+    for (int l = 1; l < hidden; ++l) {
+        const float v[3] = {h[0], h[R - 1], 0.0f};
+        layer(v, W);
+    }
+    float z = 0.0f;
+#pragma unroll
+    for (int r = 0; r < R; ++r)
+#pragma unroll 8
+        for (int k = 0; k < 32; ++k)
+            z = fmaf(__shfl_sync(0xffffffffu, h[r], k), __ldg(w + (size_t)(32 * r + k) * 4 + (lane & 3)), z);
+    z += __ldg(w + 4 * W + (lane & 3));
+    if (lane < 4)
+        reinterpret_cast<float*>(static_cast<float4*>(g.slot_out) + sample_slot(g, id, j))[lane] =
+            lane == 0 ? softplus_f32(z) : sigmoid_f32(z);
+}
+
 // HC > 0: the number of hidden layers fixed at compile time.
 template <int W, int HC, bool JIT>
-__global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
+__global__ void __launch_bounds__(kThreads, 1) k_mlp_split(const __grid_constant__ MlpArgs g) {
     const int hidden = HC > 0 ? HC : g.hidden;
     extern __shared__ __align__(1024) uint8_t smem[];
     const SplitLayout lay(W, hidden);
@@ -518,8 +598,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
                     tmem_ld_wait_regs(v);
 #pragma unroll
                     for (int i = 0; i < 8; ++i)
-                        split3(fmaxf(__uint_as_float(v[2 * i]), 0.0f), fmaxf(__uint_as_float(v[2 * i + 1]), 0.0f), wh[i],
-                               wm[i], wl[i]);
+                        split3(relu_nan(__uint_as_float(v[2 * i])), relu_nan(__uint_as_float(v[2 * i + 1])), wh[i], wm[i], wl[i]);
                     tmem_st8(a_row + col / 2, wh);
                     tmem_st8(a_row + 32u + col / 2, wm);
                     tmem_st8(a_row + 64u + col / 2, wl);
@@ -542,13 +621,24 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(MlpArgs g) {
                 tmem_ld_wait_regs(z);
             }
             if (more) store(0);
-            if (half == 0 && id_cur != 0xffffffffu) {
-                float4 o;
-                o.x = softplus_f32(__uint_as_float(z[0]) + bo.x);
-                o.y = sigmoid_f32(__uint_as_float(z[1]) + bo.y);
-                o.z = sigmoid_f32(__uint_as_float(z[2]) + bo.z);
-                o.w = sigmoid_f32(__uint_as_float(z[3]) + bo.w);
-                static_cast<float4*>(g.slot_out)[sample_slot(g, id_cur, j)] = o;
+            if (half == 0) {
+                bool nan = false;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) nan |= isnan(__uint_as_float(z[c]));
+                if (id_cur != 0xffffffffu && !nan) {
+                    float4 o;
+                    o.x = softplus_f32(__uint_as_float(z[0]) + bo.x);
+                    o.y = sigmoid_f32(__uint_as_float(z[1]) + bo.y);
+                    o.z = sigmoid_f32(__uint_as_float(z[2]) + bo.z);
+                    o.w = sigmoid_f32(__uint_as_float(z[3]) + bo.w);
+                    static_cast<float4*>(g.slot_out)[sample_slot(g, id_cur, j)] = o;
+                }
+                uint32_t redo = __ballot_sync(0xffffffffu, nan && id_cur != 0xffffffffu);
+                for (; redo; redo &= redo - 1u) {
+                    const int src = __ffs(redo) - 1;
+                    fp32_sample<W, JIT>(g, leaf, hidden, __shfl_sync(0xffffffffu, id_cur, src),
+                                        __shfl_sync(0xffffffffu, j, src));
+                }
             }
         }
         if (!ok && lane_id == 0) atomicCAS(g.err, 0, kDevErrTimeout);
@@ -578,7 +668,7 @@ cudaError_t prepare_w(int max_smem) {
 template <int W>
 cudaError_t launch_w(cudaStream_t s, const MlpArgs& a, int grid, size_t smem) {
     const bool hc = a.hidden == kHiddenFor<W>;
-    void (*kern)(MlpArgs) = a.jitter ? (hc ? k_mlp_split<W, kHiddenFor<W>, true> : k_mlp_split<W, 0, true>)
+    void (*kern)(const MlpArgs) = a.jitter ? (hc ? k_mlp_split<W, kHiddenFor<W>, true> : k_mlp_split<W, 0, true>)
                                      : (hc ? k_mlp_split<W, kHiddenFor<W>, false> : k_mlp_split<W, 0, false>);
     return launch_after(s, a.chain, kern, (unsigned)grid, (unsigned)kThreads, smem, a);
 }

@@ -127,6 +127,14 @@ void dfree(T*& p) {
     p = nullptr;
 }
 
+// Host memory to the device in the context's stream, complete on return.  Not a plain cudaMemcpy:
+// that is a copy on the legacy stream, which may still be running when the call returns
+// (pageable memory) and which kernels on a non-blocking stream do not wait for.
+cudaError_t upload(amnerf_ctx* ctx, void* dst, const void* src, size_t bytes) {
+    const cudaError_t e = cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, ctx->stream);
+    return e != cudaSuccess ? e : cudaStreamSynchronize(ctx->stream);
+}
+
 void free_ray_scratch(amnerf_ctx* ctx) {
     dfree(ctx->d_nx);
     dfree(ctx->d_xing);
@@ -298,7 +306,8 @@ amnerf_status amnerf_create(amnerf_ctx** out, int device, void* cuda_stream) {
         (e = cudaMalloc((void**)&ctx->d_offsets, sizeof(uint32_t) * (kMaxNets + 1))) != cudaSuccess ||
         (e = cudaMalloc((void**)&ctx->d_tile_off, sizeof(uint32_t) * (kMaxNets + 1))) != cudaSuccess ||
         (e = cudaMalloc((void**)&ctx->d_err, sizeof(int))) != cudaSuccess ||
-        (e = cudaMemset(ctx->d_err, 0, sizeof(int))) != cudaSuccess) {
+        (e = cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream)) != cudaSuccess ||
+        (e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) {
         amnerf_destroy(ctx);
         return e == cudaErrorMemoryAllocation ? AMNERF_E_NOMEM : AMNERF_E_CUDA;
     }
@@ -394,16 +403,15 @@ amnerf_status amnerf_build_tree(amnerf_ctx* ctx, const float* grid_host, int G, 
     dfree(ctx->d_grid);
     ctx->grid_G = 0;
     CK(cudaMalloc((void**)&ctx->d_nodes, sizeof(DevNode) * dn.size()), "tree allocation");
-    CK(cudaMemcpy(ctx->d_nodes, dn.data(), sizeof(DevNode) * dn.size(), cudaMemcpyHostToDevice), "tree upload");
+    CK(upload(ctx, ctx->d_nodes, dn.data(), sizeof(DevNode) * dn.size()), "tree upload");
     CK(cudaMalloc((void**)&ctx->d_walk, sizeof(float2) * wk.size()), "tree allocation");
-    CK(cudaMemcpy(ctx->d_walk, wk.data(), sizeof(float2) * wk.size(), cudaMemcpyHostToDevice), "tree upload");
+    CK(upload(ctx, ctx->d_walk, wk.data(), sizeof(float2) * wk.size()), "tree upload");
     CK(cudaMalloc((void**)&ctx->d_node_net, sizeof(uint16_t) * net.size()), "tree allocation");
-    CK(cudaMemcpy(ctx->d_node_net, net.data(), sizeof(uint16_t) * net.size(), cudaMemcpyHostToDevice),
-       "tree upload");
+    CK(upload(ctx, ctx->d_node_net, net.data(), sizeof(uint16_t) * net.size()), "tree upload");
     // the guidance grid stays resident for empty-space skipping
     const size_t cells = (size_t)G * G * G;
     CK(cudaMalloc((void**)&ctx->d_grid, sizeof(float) * cells), "grid allocation");
-    CK(cudaMemcpy(ctx->d_grid, grid_host, sizeof(float) * cells, cudaMemcpyHostToDevice), "grid upload");
+    CK(upload(ctx, ctx->d_grid, grid_host, sizeof(float) * cells), "grid upload");
     ctx->grid_G = G;
     for (int a = 0; a < 3; ++a) {
         ctx->grid_lo[a] = (float)bbox[a];
@@ -475,7 +483,7 @@ static amnerf_status load_impl(amnerf_ctx* ctx, const amnerf_mlp_desc* desc, int
     dfree(ctx->d_split);
     ctx->mlp_loaded = false;
     CK(cudaMalloc(&ctx->d_weights, blob.size()), "weight allocation");
-    CK(cudaMemcpy(ctx->d_weights, blob.data(), blob.size(), cudaMemcpyHostToDevice), "weight upload");
+    CK(upload(ctx, ctx->d_weights, blob.data(), blob.size()), "weight upload");
     if (m.prec == AMNERF_FP32) {
         // the same networks as split operands (k_mlp_split.cu), packed on the device from the
         // blob just uploaded; without them (shape, shared memory or device memory) the SIMT
@@ -792,7 +800,7 @@ static amnerf_status render_impl(amnerf_ctx* ctx, const float* ro, const float* 
         int herr = 0;
         CK(cudaMemcpy(&herr, ctx->d_err, sizeof herr, cudaMemcpyDeviceToHost), "status copy");
         if (herr) {
-            cudaMemset(ctx->d_err, 0, sizeof(int));
+            cudaMemsetAsync(ctx->d_err, 0, sizeof(int), s);
             return fail(ctx, device_status(herr), "device status word set");
         }
     }
@@ -948,10 +956,10 @@ amnerf_status amnerf_proposal_set(amnerf_ctx* ctx, const float* params, const fl
         CK(cudaMalloc((void**)&ctx->d_prop, sizeof(float) * (5 * (size_t)np + 1)), "proposal allocation");
         CK(prepare_proposal(&ctx->prop_grid), "proposal kernel setup");
     }
-    CK(cudaMemset(ctx->d_prop, 0, sizeof(float) * (5 * (size_t)np + 1)), "memset");
-    CK(cudaMemcpy(prop_params(ctx), params, sizeof(float) * np, cudaMemcpyHostToDevice), "proposal upload");
-    if (m) CK(cudaMemcpy(prop_m(ctx), m, sizeof(float) * np, cudaMemcpyHostToDevice), "proposal upload");
-    if (v) CK(cudaMemcpy(prop_v(ctx), v, sizeof(float) * np, cudaMemcpyHostToDevice), "proposal upload");
+    CK(cudaMemsetAsync(ctx->d_prop, 0, sizeof(float) * (5 * (size_t)np + 1), ctx->stream), "memset");
+    CK(upload(ctx, prop_params(ctx), params, sizeof(float) * np), "proposal upload");
+    if (m) CK(upload(ctx, prop_m(ctx), m, sizeof(float) * np), "proposal upload");
+    if (v) CK(upload(ctx, prop_v(ctx), v, sizeof(float) * np), "proposal upload");
     ctx->prop_step = step;
     ctx->prop_loaded = true;
     return AMNERF_OK;
@@ -1140,7 +1148,7 @@ amnerf_status amnerf_sync(amnerf_ctx* ctx) {
     int herr = 0;
     CK(cudaMemcpy(&herr, ctx->d_err, sizeof herr, cudaMemcpyDeviceToHost), "status copy");
     if (herr) {
-        cudaMemset(ctx->d_err, 0, sizeof(int));
+        cudaMemsetAsync(ctx->d_err, 0, sizeof(int), ctx->stream);
         return fail(ctx, device_status(herr), "device status word set");
     }
     return AMNERF_OK;

@@ -491,7 +491,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(const __grid_constant
             __syncwarp();
             if (lane_id == 0) mbar_arrive(bar_a);
         };
-        float x[3], d[3];
+        float x[3] = {0.f, 0.f, 0.f}, d[3] = {0.f, 0.f, 0.f};
         // this half's eight words (column pairs) of a chunk of the layer-0 input, split
         uint32_t wh[8], wm[8], wl[8];
         // pair p < 42: sine and cosine
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_mlp_split(const __grid_constant
                 uint32_t redo = __ballot_sync(0xffffffffu, nan && id_cur != 0xffffffffu);
                 for (; redo; redo &= redo - 1u) {
                     const int src = __ffs(redo) - 1;
-                    fp32_sample<W, JIT>(g, leaf, hidden, __shfl_sync(0xffffffffu, id_cur, src),
+                    fp32_sample<W, JIT>(g, cur, hidden, __shfl_sync(0xffffffffu, id_cur, src),
                                         __shfl_sync(0xffffffffu, j, src));
                 }
             }

@@ -81,46 +81,6 @@ __device__ __forceinline__ void prop_features(const float o[3], const float d[3]
         for (int a = 0; a < 3; ++a) sincospif(d[a] * (float)(1 << k), &x[(66 + 6 * k + a) * S], &x[(69 + 6 * k + a) * S]);
 }
 
-// Forward pass from features in shared memory row xr (stride 1) with parameters in
-// shared memory P; h1, h2 post-ReLU, q softmax.
-__device__ __forceinline__ void prop_forward(const float* __restrict__ P, const float* xr, float* h1, float* h2,
-                                             float* q) {
-#pragma unroll
-    for (int o = 0; o < PH; ++o) h1[o] = P[OFF_B1 + o];
-    for (int f = 0; f < PIN; ++f) {
-        const float v = xr[f];
-#pragma unroll
-        for (int o = 0; o < PH; ++o) h1[o] = fmaf(P[OFF_W1 + o * PIN + f], v, h1[o]);
-    }
-#pragma unroll
-    for (int o = 0; o < PH; ++o) h1[o] = fmaxf(h1[o], 0.0f);
-#pragma unroll
-    for (int o = 0; o < PH; ++o) {
-        float acc = P[OFF_B2 + o];
-#pragma unroll
-        for (int i = 0; i < PH; ++i) acc = fmaf(P[OFF_W2 + o * PH + i], h1[i], acc);
-        h2[o] = fmaxf(acc, 0.0f);
-    }
-    float m = -INFINITY;
-#pragma unroll
-    for (int o = 0; o < PO; ++o) {
-        float acc = P[OFF_B3 + o];
-#pragma unroll
-        for (int i = 0; i < PH; ++i) acc = fmaf(P[OFF_W3 + o * PH + i], h2[i], acc);
-        q[o] = acc;
-        m = fmaxf(m, acc);
-    }
-    float s = 0.0f;
-#pragma unroll
-    for (int o = 0; o < PO; ++o) {
-        q[o] = expf(q[o] - m);
-        s += q[o];
-    }
-    const float inv = 1.0f / s;
-#pragma unroll
-    for (int o = 0; o < PO; ++o) q[o] *= inv;
-}
-
 // ---- inference ---------------------------------------------------------------------
 // Persistent CTAs over tiles of kRays rays.  Each layer is a (kRays x 32) x K FP32
 // product formed from shared memory: activations are stored feature-major

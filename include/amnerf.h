@@ -263,6 +263,12 @@ AMNERF_API amnerf_status amnerf_get_tree(amnerf_ctx *ctx, amnerf_node *nodes_out
  * The library repacks the weights into the layout of desc->prec (FP32 transposed
  * tiles, BF16 or E4M3 tcgen05 core-matrix tiles; E4M3 per-leaf, per-layer,
  * per-output-channel scales s = max|W_row| / 448).  Synchronous.
+ * Device memory per network of 4 x 64: 46 KB in BF16, 30 KB in E4M3.  FP32 networks
+ * with lx = 10, ld = 4 are held twice: the transposed tiles (74 KB: calibration, and samples
+ * whose activations overflow) and, where the shared memory can hold them, their three-part
+ * split for the tensor cores (123 KB; 1 GB for 8191 networks).  If the second copy cannot be
+ * allocated the load succeeds without it and renders use the FP32 lanes (about six times
+ * slower, the same accuracy).
  * Errors: E_NOTREE, E_INVAL (shape unsupported or n_leaves neither count), E_NOMEM. */
 AMNERF_API amnerf_status amnerf_load_mlps(amnerf_ctx *ctx, const amnerf_mlp_desc *desc, int n_leaves,
                                const float *weights_host);
@@ -361,7 +367,10 @@ AMNERF_API amnerf_status amnerf_sync(amnerf_ctx *ctx);
  * the call returns AMNERF_E_TIMEOUT and the context stays usable. */
 AMNERF_API amnerf_status amnerf_selftest_wait(amnerf_ctx *ctx, uint64_t cycles);
 
-/* Record per-stage CUDA-event timing in later renders (amnerf_stats.ms). */
+/* Record per-stage CUDA-event timing in later renders (amnerf_stats.ms).  The stages of a
+ * timed render are ordinary launches, one after the other; those of an untimed small batch
+ * overlap (each may start before the one before has ended), so that its stages' times sum to
+ * more than its untimed call takes. */
 AMNERF_API amnerf_status amnerf_set_timing(amnerf_ctx *ctx, int enable);
 
 /* Group crossings by leaf without allocating anything (no counterpart in the paper;

@@ -60,8 +60,11 @@ __device__ __forceinline__ float jit_fraction(uint64_t seed, uint64_t key, int k
 // ---- dependent launches ------------------------------------------------------------------
 // A grid launched after another with `pdl` may start once every CTA of that one has called
 // grid_launch (or ended); grid_wait then waits until it has ended and its writes are visible.
-// What such a predecessor wrote is read after grid_wait with loads that go to L2 (__ldcg,
-// cp.async): this grid may have started before it was written.
+// What such a predecessor wrote is read after grid_wait only, and not with ld.global.nc, since
+// this grid may have started before it was written: with __ldcg, which goes to L2, or with
+// cp.async.ca, which keeps lines in L1.  The latter is safe because no grid of a chain touches
+// those lines (crossing ids and intervals) before its own grid_wait, and because a chain starts
+// with an ordinary launch, which leaves no older copy of them in an L1.
 __device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

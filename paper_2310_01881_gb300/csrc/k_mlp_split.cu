@@ -6,19 +6,20 @@
 // BF16 value 8 and FP32's exponents, so v = h + m + l with h = bf16(v), m = bf16(v - h),
 // l = bf16(v - h - m) is exact (below about 2^-110, where parts become subnormal, up to an
 // absolute 2^-133).  A product of two split values is taken as the six largest of its nine
-// partial products -- h h, h m, m h, m m, h l, l h; the three left out are below
-// 2^-26 of it -- with the FP32 accumulator of the MMA.  That is the SIMT path's precision,
-// not a lower one: no operand or partial sum has fewer bits than FP32's own rounding.  The
-// tensor cores' accumulation truncates where FP32 arithmetic rounds to nearest, so each
-// layer adds its small products first (the accumulator then is 2^-8 of the sum, and so is
-// what a truncation drops), then the bias, and the h h products last: 5 or 6 accumulations
-// at full size against 64 to 90 roundings of an FP32 chain.
+// partial products -- h h, h m, m h, m m, h l, l h.  |m| is at most 2^-8 and |l| 2^-17 of a
+// value, so the three left out (m l, l m, l l) are at most about 2^-24 of the product, as large
+// as the one rounding that an FP32 product has, and mostly far smaller.  The tensor cores'
+// accumulation truncates where FP32 arithmetic rounds to nearest, so each layer adds its small
+// products first (the accumulator then is 2^-8 of the sum, and so is what a truncation drops),
+// then the bias, and the h h products last: 5 or 6 accumulations at full size against 64 to 90
+// roundings of an FP32 chain.  That this is the SIMT path's precision, and not a lower one, is
+// measured:
 //
-// Measured against 64 bits (relative 2-norm of the pixels' error, one 800 x 800 view):
+// Against 64 bits (relative 2-norm of the pixels' error, one 800 x 800 view):
 // 9.1e-7 with the SIMT kernel, 9.1e-7 here; the networks' own outputs, on the same sample
-// positions: 4.3e-8 (sigma) and 5.6e-8 (rgb) with the SIMT kernel, 4.3e-8 and 5.6e-8 here
-// (256 networks of 4 x 64), 2.6e-7 and 7.0e-7 against 2.5e-7 and 2.7e-7 with weights three
-// times as large; the largest single error is lower in every scene and shape measured.
+// positions (256 networks of 4 x 64, 48 x 48 rays): 4.9e-8 (sigma) and 6.4e-8 (rgb) with the
+// SIMT kernel, 4.7e-8 and 6.0e-8 here; with weights three times as large 2.5e-7 and 7.4e-7
+// with the SIMT kernel, 2.6e-7 and 2.8e-7 here; the largest single error is lower in each.
 //
 // What bounds it: a 4 x 64 tile takes 135 MMAs, about 4 400 cycles of the tensor pipe, and
 // its rows about 2 500 instruction issues per SM sub-partition (nine instructions per split
@@ -40,6 +41,11 @@
 // The samples of a crossing share their direction's features (eight lanes compute a pair
 // each and exchange them, at 8 samples per crossing or more).  While the head runs, a group
 // encodes the first chunk of its next tile.  Every wait is bounded.
+//
+// Overflow: the parts of an infinity do not multiply as it does, so an activation that is
+// infinite or NaN gets a NaN among its parts, and a sample whose head sums are NaN is computed
+// again in FP32 (fp32_sample).  Its cost where nothing overflows: none measurable at 4 x 64
+// (6.16 and 6.14 ms per view without and with it), 2 % at eight layers of 32.
 //
 // Kept on the SIMT kernel: calibration (per-layer input maxima), other encodings than
 // lx = 10, ld = 4, and networks whose split weights do not fit the shared memory.

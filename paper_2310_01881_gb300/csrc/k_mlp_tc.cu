@@ -198,7 +198,7 @@ constexpr uint32_t kA0Col8 = 16;  // E4M3: first A column of the layer-0 input
 
 // Registers per thread: 128 (groups + 1) threads are launched with 96 each; the compute
 // warpgroups take more and leave the last one the rest (at four groups the whole launch:
-// 4 x 112 + 32 = 5 x 96; fewer groups ask for less than they were launched with).
+// 4 x 104 + 64 = 5 x 96; fewer groups ask for less than they were launched with).
 constexpr int kComputeRegs = 104, kAuxRegs = 64;
 static_assert(kMaxGroups * kComputeRegs + kAuxRegs <= (kMaxGroups + 1) * 96 && kComputeRegs - 96 <= 96 - kAuxRegs,
               "the split draws on the launch's registers");
@@ -214,7 +214,9 @@ static_assert(kMaxGroups * kComputeRegs + kAuxRegs <= (kMaxGroups + 1) * 96 && k
 // HC > 0: the number of hidden layers fixed at compile time, so the layer loop is
 // unrolled and every layout offset is a constant (about 12 % faster on the 4 x 64
 // network); HC = 0 reads it from the arguments.  The shapes of the workloads here
-// (4 x 64 and 2 x 32) are instantiated with HC set.
+// (4 x 64 and 2 x 32) are instantiated with HC set and spill no register; at HC = 0 the words
+// of the next tile's input that live across the layer loop are spilled: 104 bytes per thread
+// in the 64-wide BF16 kernel (84 with jitter), 68 in the per-row E4M3 one, 8 in the others.
 template <int W>
 constexpr int kHiddenFor = W == 64 ? 4 : 2;
 
@@ -741,8 +743,8 @@ __global__ void __launch_bounds__(128 * (kMaxGroups + 1), 1) k_mlp_tc(MlpArgs g,
                     } else {
                         // the row's activations and their maximum, 16 columns at a time and
                         // back into D, then scaled by it: the row does not fit the registers
-                        // beside the rest (88 bytes spilled; without them, and with the encoding in
-                        // two passes, 640 000 rays take 2.68 ms against 3.02)
+                        // beside the rest (4 x 64: 88 bytes spilled; without them, and with the
+                        // encoding in two passes, 640 000 rays take 2.68 ms against 3.02)
                         float m = 0.0f;
 #pragma unroll
                         for (int h = 0; h < W / 16; ++h) {

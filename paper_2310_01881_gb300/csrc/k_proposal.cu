@@ -587,14 +587,16 @@ __device__ __forceinline__ uint32_t batch_ray(uint64_t seed, uint64_t s, uint32_
 // k_prop_grad leaves one partial gradient per CTA, k_prop_reduce sums the partials in a
 // fixed order and updates the parameters (no atomics: a step's result does not vary).
 //
-// What bounds it: a step is 0.3 GFLOP, so latency.  With one thread per ray (64 CTAs of 128
-// threads, each thread walking its ray's 6 000 multiply-adds alone) a step of 8192 rays took
-// 98 us; with 64 rays per CTA of 512 threads, every layer and contraction spread over all of
-// them from shared memory, 25 us (24 steps 2.36 -> 0.60 ms).  Rows of 68 floats keep the 16-byte loads of
-// neighbouring rows on different banks.  The next step's launch overlaps its ray loads and
-// encodings with the update (programmatic dependent launch).
+// What bounds it: a step is 0.3 GFLOP, so latency, first that of shared-memory loads.  With one
+// thread per ray (64 CTAs of 128 threads, each thread walking its ray's 6 000 multiply-adds
+// alone) a step of 8192 rays took 98 us; with 64 rays per CTA of 512 threads, every layer and
+// contraction spread over all of them from shared memory, 25 us (24 steps 2.36 -> 0.60 ms).
+// Rows of 68 floats keep the 16-byte loads of neighbouring rows on different banks.  The next
+// step's launch overlaps its ray loads and encodings with the update (programmatic dependent
+// launch).
 constexpr int kGRays = 64, kGThreads = 512, kGLd = 68;
-constexpr int kPartCtas = 304;       // at most (two per SM); each takes every kPartCtas-th tile of 64 rays
+constexpr int kPartCtas = 304;       // at most (two rounds of one CTA per SM, which its registers admit); each
+                                     // takes every kPartCtas-th tile of 64 rays
 constexpr int kPartStride = 6144;  // floats per partial: the gradient, then the loss
 static_assert(NPAR < kPartStride, "partial gradient");
 struct GradSmem {

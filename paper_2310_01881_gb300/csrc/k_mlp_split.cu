@@ -45,7 +45,9 @@
 // Overflow: the parts of an infinity do not multiply as it does, so an activation that is
 // infinite or NaN gets a NaN among its parts, and a sample whose head sums are NaN is computed
 // again in FP32 (fp32_sample).  Its cost where nothing overflows: none measurable at 4 x 64
-// (6.16 and 6.14 ms per view without and with it), 2 % at eight layers of 32.
+// (6.16 and 6.14 ms per view without and with it), 2 % at eight layers of 32; where every
+// sample overflows an 800 x 800 view takes 161 ms (35 on the SIMT kernel).  A sum whose partial
+// sums overflow in one order of its terms and not in another may still come out either way.
 //
 // Kept on the SIMT kernel: calibration (per-layer input maxima), other encodings than
 // lx = 10, ld = 4, and networks whose split weights do not fit the shared memory.
